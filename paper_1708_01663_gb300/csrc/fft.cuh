@@ -38,64 +38,87 @@ template <bool INV, typename C> __device__ __forceinline__ C f_rot(C a) {
   return INV ? cx<C>::make(-a.y, a.x) : cx<C>::make(a.y, -a.x);
 }
 
+// Packed complex64 arithmetic (PK): the sm_100 family adds or multiply-adds the two floats of an aligned register
+// pair in one instruction.  The FP32 rate is the same (37.5 against 36.8 T sums/s measured), but the pair takes one
+// issue slot instead of two, which is what the two-stage kernels lack (issue 60 to 66 % of cycles, FP32 pipe 35 to
+// 53 %): the P = 512 pass of 64 transmitters went from 93.6 to 89.9 us, P = 256 (8) from 11.1 to 10.4 us.  The
+// three-stage kernels keep scalar sums: the pairs cost them more in scheduling (P = 512 columns, 512 threads: pass
+// 107 -> 112 us) than the slots gain.  Each half rounds as the scalar instruction does.  A product with -+i swaps
+// the halves, which no packed instruction does, so those sums are scalar everywhere, as are FP64 and the host build.
+template <bool PK, typename C> __device__ __forceinline__ C p_add(C a, C b) {
+#if defined(__CUDA_ARCH__)
+  if constexpr (PK) return __fadd2_rn(a, b);
+#endif
+  return f_add(a, b);
+}
+// a + s b, s a constant
+template <bool PK, typename C, typename R> __device__ __forceinline__ C p_axpy(R s, C b, C a) {
+#if defined(__CUDA_ARCH__)
+  if constexpr (PK) return __ffma2_rn(make_float2(s, s), b, a);
+#endif
+  return cx<C>::make(a.x + s * b.x, a.y + s * b.y);
+}
+template <bool PK, typename C> __device__ __forceinline__ C p_sub(C a, C b) {
+#if defined(__CUDA_ARCH__)
+  if constexpr (PK) return p_axpy<PK>(-1.f, b, a);
+#endif
+  return f_sub(a, b);
+}
+// a + b times (-i, or +i for the inverse), and a minus it
+template <bool INV, typename C> __device__ __forceinline__ C f_addrot(C a, C b) {
+  return INV ? cx<C>::make(a.x - b.y, a.y + b.x) : cx<C>::make(a.x + b.y, a.y - b.x);
+}
+template <bool INV, typename C> __device__ __forceinline__ C f_subrot(C a, C b) { return f_addrot<!INV>(a, b); }
+
 template <bool INV, typename C> __device__ __forceinline__ void dft2(C& a0, C& a1) {
   C t = a0;
   a0 = f_add(t, a1);
   a1 = f_sub(t, a1);
 }
 
-template <bool INV, typename C> __device__ __forceinline__ void dft4(C& a0, C& a1, C& a2, C& a3) {
-  C t0 = f_add(a0, a2), t1 = f_sub(a0, a2);
-  C t2 = f_add(a1, a3), t3 = f_rot<INV>(f_sub(a1, a3));
-  a0 = f_add(t0, t2);
-  a1 = f_add(t1, t3);
-  a2 = f_sub(t0, t2);
-  a3 = f_sub(t1, t3);
+template <bool INV, bool PK = false, typename C> __device__ __forceinline__ void dft4(C& a0, C& a1, C& a2, C& a3) {
+  const C t0 = p_add<PK>(a0, a2), t1 = p_sub<PK>(a0, a2);
+  const C t2 = p_add<PK>(a1, a3), d = p_sub<PK>(a1, a3);
+  a0 = p_add<PK>(t0, t2);
+  a1 = f_addrot<INV>(t1, d);
+  a2 = p_sub<PK>(t0, t2);
+  a3 = f_subrot<INV>(t1, d);
+}
+
+// the last layer of a radix-8 DFT from the radix-4 DFTs of its even (e) and odd (o) inputs, joined by w8^k:
+// w8 = (1 -+ i)/sqrt2, w8^2 = -+i, w8^3 = (-1 -+ i)/sqrt2
+template <bool INV, bool PK, typename C> __device__ __forceinline__ void dft8_join(C* v, const C* e, const C* o) {
+  typedef typename cx<C>::R R;
+  const R h = (R)0.70710678118654752440;
+  // sqrt2 w8 o1 and -sqrt2 w8^3 o3
+  const C p = INV ? cx<C>::make(o[1].x - o[1].y, o[1].x + o[1].y) : cx<C>::make(o[1].x + o[1].y, o[1].y - o[1].x);
+  const C q = INV ? cx<C>::make(o[3].x + o[3].y, o[3].y - o[3].x) : cx<C>::make(o[3].x - o[3].y, o[3].x + o[3].y);
+  v[0] = p_add<PK>(e[0], o[0]);
+  v[4] = p_sub<PK>(e[0], o[0]);
+  v[1] = p_axpy<PK>(h, p, e[1]);
+  v[5] = p_axpy<PK>(-h, p, e[1]);
+  v[2] = f_addrot<INV>(e[2], o[2]);
+  v[6] = f_subrot<INV>(e[2], o[2]);
+  v[3] = p_axpy<PK>(-h, q, e[3]);
+  v[7] = p_axpy<PK>(h, q, e[3]);
 }
 
 // radix-8 = two radix-4 DFTs (even / odd inputs) joined by w8^k, k = 0..3
-template <bool INV, typename C> __device__ __forceinline__ void dft8(C* v) {
-  typedef typename cx<C>::R R;
-  C e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
-  C o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
-  dft4<INV>(e0, e1, e2, e3);
-  dft4<INV>(o0, o1, o2, o3);
-  const R h = (R)0.70710678118654752440;
-  // w8 = (1 -+ i)/sqrt2 ; w8^2 = -+i ; w8^3 = (-1 -+ i)/sqrt2
-  C w1o = INV ? cx<C>::make(h * (o1.x - o1.y), h * (o1.x + o1.y)) : cx<C>::make(h * (o1.x + o1.y), h * (o1.y - o1.x));
-  C w2o = f_rot<INV>(o2);
-  C w3o = INV ? cx<C>::make(-h * (o3.x + o3.y), h * (o3.x - o3.y)) : cx<C>::make(h * (o3.y - o3.x), -h * (o3.x + o3.y));
-  v[0] = f_add(e0, o0);
-  v[4] = f_sub(e0, o0);
-  v[1] = f_add(e1, w1o);
-  v[5] = f_sub(e1, w1o);
-  v[2] = f_add(e2, w2o);
-  v[6] = f_sub(e2, w2o);
-  v[3] = f_add(e3, w3o);
-  v[7] = f_sub(e3, w3o);
+template <bool INV, bool PK = false, typename C> __device__ __forceinline__ void dft8(C* v) {
+  C e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+  dft4<INV, PK>(e[0], e[1], e[2], e[3]);
+  dft4<INV, PK>(o[0], o[1], o[2], o[3]);
+  dft8_join<INV, PK>(v, e, o);
 }
 
 // radix-8 DFT of inputs whose upper half v[4..7] is zero (the first stage of a
 // transform of a zero-padded sequence, padding >= half the length): each
 // radix-4 half sees two non-zero inputs, so its first butterfly layer is a
 // copy: DFT4(a, b, 0, 0) = (a + b, a + rot(b), a - b, a - rot(b)).
-template <bool INV, typename C> __device__ __forceinline__ void dft8_lo(C* v) {
-  typedef typename cx<C>::R R;
-  const C re1 = f_rot<INV>(v[2]), ro1 = f_rot<INV>(v[3]);
-  C e0 = f_add(v[0], v[2]), e1 = f_add(v[0], re1), e2 = f_sub(v[0], v[2]), e3 = f_sub(v[0], re1);
-  C o0 = f_add(v[1], v[3]), o1 = f_add(v[1], ro1), o2 = f_sub(v[1], v[3]), o3 = f_sub(v[1], ro1);
-  const R h = (R)0.70710678118654752440;
-  C w1o = INV ? cx<C>::make(h * (o1.x - o1.y), h * (o1.x + o1.y)) : cx<C>::make(h * (o1.x + o1.y), h * (o1.y - o1.x));
-  C w2o = f_rot<INV>(o2);
-  C w3o = INV ? cx<C>::make(-h * (o3.x + o3.y), h * (o3.x - o3.y)) : cx<C>::make(h * (o3.y - o3.x), -h * (o3.x + o3.y));
-  v[0] = f_add(e0, o0);
-  v[4] = f_sub(e0, o0);
-  v[1] = f_add(e1, w1o);
-  v[5] = f_sub(e1, w1o);
-  v[2] = f_add(e2, w2o);
-  v[6] = f_sub(e2, w2o);
-  v[3] = f_add(e3, w3o);
-  v[7] = f_sub(e3, w3o);
+template <bool INV, bool PK = false, typename C> __device__ __forceinline__ void dft8_lo(C* v) {
+  const C e[4] = {p_add<PK>(v[0], v[2]), f_addrot<INV>(v[0], v[2]), p_sub<PK>(v[0], v[2]), f_subrot<INV>(v[0], v[2])};
+  const C o[4] = {p_add<PK>(v[1], v[3]), f_addrot<INV>(v[1], v[3]), p_sub<PK>(v[1], v[3]), f_subrot<INV>(v[1], v[3])};
+  dft8_join<INV, PK>(v, e, o);
 }
 
 // cos(pi m / 16) and sin(pi m / 16) for 0 <= m <= 16 (decimal expansions).
@@ -134,16 +157,16 @@ template <bool INV> __device__ __forceinline__ void dft16(float2* v) {
     e[i] = v[2 * i];
     o[i] = v[2 * i + 1];
   }
-  dft8<INV>(e);
-  dft8<INV>(o);
+  dft8<INV, true>(e);
+  dft8<INV, true>(o);
   const float2 t0 = o[0], t1 = mul_w32<INV, 2>(o[1]), t2 = mul_w32<INV, 4>(o[2]), t3 = mul_w32<INV, 6>(o[3]),
                t4 = mul_w32<INV, 8>(o[4]), t5 = mul_w32<INV, 10>(o[5]), t6 = mul_w32<INV, 12>(o[6]),
                t7 = mul_w32<INV, 14>(o[7]);
   const float2 t[8] = {t0, t1, t2, t3, t4, t5, t6, t7};
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    v[k] = f_add(e[k], t[k]);
-    v[k + 8] = f_sub(e[k], t[k]);
+    v[k] = p_add<true>(e[k], t[k]);
+    v[k + 8] = p_sub<true>(e[k], t[k]);
   }
 }
 
@@ -179,8 +202,8 @@ template <bool INV> __device__ __forceinline__ void dft32(float2* v) {
   mul_w32_ramp<INV>(o);
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
-    v[k] = f_add(e[k], o[k]);
-    v[k + 16] = f_sub(e[k], o[k]);
+    v[k] = p_add<true>(e[k], o[k]);
+    v[k + 16] = p_sub<true>(e[k], o[k]);
   }
 }
 
@@ -214,8 +237,8 @@ template <bool INV> __device__ __forceinline__ void dft16_lo(float2* v) {
   b[5] = mul_w32<INV, 10>(v[5]);
   b[6] = mul_w32<INV, 12>(v[6]);
   b[7] = mul_w32<INV, 14>(v[7]);
-  dft8<INV>(a);
-  dft8<INV>(b);
+  dft8<INV, true>(a);
+  dft8<INV, true>(b);
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
     v[2 * m] = a[m];
@@ -227,11 +250,12 @@ template <bool INV> __device__ __forceinline__ void dft16_lo(float2* v) {
 template <int N, bool INV> __device__ __forceinline__ void dft_n(float2* v) {
   if constexpr (N == 32) dft32<INV>(v);
   else if constexpr (N == 16) dft16<INV>(v);
-  else dft8<INV>(v);
+  else dft8<INV, true>(v);
 }
 template <int N, bool INV> __device__ __forceinline__ void dft_n_lo(float2* v) {
   if constexpr (N == 32) dft32_lo<INV>(v);
-  else dft16_lo<INV>(v);
+  else if constexpr (N == 16) dft16_lo<INV>(v);
+  else dft8_lo<INV, true>(v);
 }
 
 template <int R, bool INV, typename C> __device__ __forceinline__ void dft_r(C* v) {
