@@ -188,7 +188,7 @@ static void free_ctx(cisor_ctx* c) {
   if (c->loop_item) cudaFree(c->loop_item);
   if (c->loop_count) cudaFree(c->loop_count);
   if (c->h_loop_count) cudaFreeHost(c->h_loop_count);
-  void* dev[] = {c->ghat, c->tw, c->twst, c->H, c->u_in, c->R, c->r, c->rhat, c->p, c->v, c->s, c->tv, c->b, c->u,
+  void* dev[] = {c->ghat, c->gplane, c->tw, c->twst, c->H, c->u_in, c->R, c->r, c->rhat, c->p, c->v, c->s, c->tv, c->b, c->u,
                  c->vadj, c->z, c->gz, c->f, c->fz, c->grad, c->work_n, c->Y, c->w, c->yobs, c->sense_part,
                  c->part, c->scal, c->active, c->iters, c->txflag, c->dsum, c->sparams, c->tv_z,
                  c->tv_r0, c->tv_r1, c->tv_p, c->rx_mask, c->tva0, c->tva1, c->vbuf, c->f_ck, c->Ht};
@@ -328,6 +328,7 @@ cisor_status cisor_create(cisor_ctx** out, const cisor_geometry* g, void* stream
   const size_t TM = (size_t)c->T * c->M * sizeof(float2);
   const size_t Pd = (size_t)P * P * (d == 3 ? P : 1);
   ALLOC(c->ghat, sizeof(float2) * Pd);
+  if (conv3_ok(d, P)) ALLOC(c->gplane, sizeof(float2) * conv3_ghat_elems(P));
   ALLOC(c->tw, sizeof(float2) * P);
   ALLOC(c->twst, sizeof(float2) * 2 * 512);
   ALLOC(c->H, (size_t)c->M * c->Nf * sizeof(float2));
@@ -835,7 +836,12 @@ cisor_status cisor_autotune(cisor_ctx* c, int reps, int* cols_nt_out) {
   CISOR_CUDA(cudaEventCreate(&e1));
   int variants[4] = {512, 256, 0, 0};
   int nvar = 2;
-  if (two_stage_ok(c)) variants[nvar++] = COLS_TWO_STAGE;
+  if (conv3_ok(c->dim, c->P)) {  // the plane pass has no column kernels: the shape in use stays
+    variants[0] = c->cols_nt;
+    nvar = 1;
+  } else if (two_stage_ok(c)) {
+    variants[nvar++] = COLS_TWO_STAGE;
+  }
   if (conv_fused_ok(c)) variants[nvar++] = COLS_CLUSTER;
   // transmitter chunks whose FFT intermediate takes about 16, 32 or 48 MB (L2 is 126 MB), and no chunking
   const int ntr = c->T * c->ncomp;
@@ -846,7 +852,7 @@ cisor_status cisor_autotune(cisor_ctx* c, int reps, int* cols_nt_out) {
     const long long k = ((long long)mb << 20) / rbytes;
     if (k >= 1 && k < ntr && (nch == 1 || k != chunks[nch - 1])) chunks[nch++] = (int)k;
   }
-  int best = 512, best_chunk = 0;
+  int best = variants[0], best_chunk = 0;
   float best_ms = 1e30f;
   cisor_status st = CISOR_OK;
   for (int v = 0; v < nvar && st == CISOR_OK; ++v)

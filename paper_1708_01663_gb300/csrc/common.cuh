@@ -5,8 +5,10 @@
 //   f           [n, n] / [n, n, n]                   complex64
 //   R (scratch) [T, n, P] (2D): the padded field after the x FFT; only the n
 //               non-zero rows of the P x P padded image are kept.
-//               [T, n, P, P] (3D): z slabs of the padded field after the x
-//               and y FFTs; only the n non-zero z slabs are kept.
+//               [T, P, n, n] (3D, P <= 128): the field after the x FFT, as
+//               one (z, y) plane per x frequency.
+//               [T, n, P, P] (3D, P = 256): z slabs of the padded field after
+//               the x and y FFTs; only the n non-zero z slabs are kept.
 //   ghat        [P^d]    complex64: spectrum of the circulant embedding of
 //               G (Sec. II, Eq. 3), pre-scaled by 1/P^d for the inverse FFTs
 //   H           [M, N]      complex64 (Eq. 2)
@@ -91,7 +93,7 @@ struct cisor_ctx {
   int ncomp;              // field components: 1 (scalar), 3 (vectorial model of the appendix)
   long long Nf;           // field length per transmitter: ncomp * N
   int nrows;              // x rows per field: n (2D), n^2 (3D)
-  long long rslab;        // R offset between z slabs (3D: P^2)
+  long long rslab;        // R offset between z slabs (3D, P = 256: P^2)
   long long rtstride;     // R elements per transmitter
   double delta, wavelength, eps_b, k, kb;
   std::vector<double> tx_angles, rx_pos;  // 2D: [T] angles, [M, 2]; 3D: [T, 3] directions, [M, 3];
@@ -103,6 +105,7 @@ struct cisor_ctx {
   cudaEvent_t ev_a, ev_b;
   // tables
   float2* ghat;   // [P^d], scaled by 1/P^d
+  float2* gplane; // one eighth of ghat in the order of the 3D plane pass (conv3d.cu; null elsewhere)
   float2* tw;     // [P] exp(-2 pi i m / P)
   float2* twst;   // [2][512] stage twiddle tables of the forward / reversed FFT plans
   float2* H;      // [M, N]
@@ -257,11 +260,18 @@ int conv_fused_pass(cisor_ctx* c, const ConvOp& op, int dk, cudaError_t* e);
 enum { EPI_MATVEC = 0, EPI_RESID = 1, EPI_CONV_ADD = 2 };
 cisor_status conv_pass(cisor_ctx* c, const ConvOp& op);
 cisor_status conv_init(int P);
-int conv_rows_per_block(int P);
+int conv_rows_per_block(int dim, int P);
 // Fills nrows, rslab, rtstride and nblk from dim, n, P.
 void conv_geometry(cisor_ctx* c);
 long long conv_scratch_elems(int dim, int n, int P);  // R elements per transmitter
-int conv_kernels_per_pass(int dim);
+int conv_kernels_per_pass(int dim, int P);
+// conv3d.cu: the three-kernel plane pass of 3D grids with P = 64 or 128
+bool conv3_ok(int dim, int P);
+int conv3_rows_per_block();
+cisor_status conv3_init(int P);
+size_t conv3_ghat_elems(int P);            // elements of c->gplane
+cisor_status conv3_tables(cisor_ctx* c);   // c->gplane from c->ghat
+cisor_status conv3_pass(cisor_ctx* c, const ConvOp& op);
 
 // solver.cu
 cisor_status solve_batch(cisor_ctx* c, int adjoint, const float2* f, const float2* b, float2* x,

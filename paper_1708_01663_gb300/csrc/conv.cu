@@ -15,9 +15,11 @@
 //                the epilogue: A x = x - G(f x), A^H x = x - conj(f) G^H x,
 //                the residual b - A x, or G^H v + z; plus up to three
 //                per-transmitter inner products (FP32 trees).
-// A 3D pass (R is [T, n, P, P]: the n non-zero z slabs of the padded volume)
-// is five kernels: rows_fwd over the n^2 x rows; cols in forward-only mode
-// along y (n inputs, P outputs per column, in each z slab); cols with the
+// A 3D pass with P = 64 or 128 is the three kernels of conv3d.cu.  With P = 256,
+// whose half-transformed planes do not fit an SM's shared memory (n P values of
+// 8 bytes), R is [T, n, P, P] (the n non-zero z slabs of the padded volume) and
+// the pass is five kernels: rows_fwd over the n^2 x rows; cols in forward-only
+// mode along y (n inputs, P outputs per column, in each z slab); cols with the
 // spectrum product along z (stride P^2; n of the P z planes kept); cols in
 // inverse-only mode along y (P inputs, n kept); rows_inv.
 // ghat is pre-scaled by 1/P^d, so the inverse transforms are unnormalised.
@@ -35,22 +37,22 @@ template <int P> struct ConvCfg {
   template <int NT> struct Col { static constexpr int W = NT / NTF; };  // columns per CTA, column pass
 };
 
-int conv_rows_per_block(int P) { return 2048 / P; }
+int conv_rows_per_block(int dim, int P) { return conv3_ok(dim, P) ? conv3_rows_per_block() : 2048 / P; }
 
 void conv_geometry(cisor_ctx* c) {
   const int n = c->n, P = c->P;
   c->nrows = c->dim == 3 ? n * n : n;
   c->rslab = c->dim == 3 ? (long long)P * P : (long long)n * P;
   c->rtstride = conv_scratch_elems(c->dim, n, P);
-  const int RB = conv_rows_per_block(P);
+  const int RB = conv_rows_per_block(c->dim, P);
   c->nblk = (c->nrows + RB - 1) / RB;
 }
 
 long long conv_scratch_elems(int dim, int n, int P) {
-  return dim == 3 ? (long long)n * P * P : (long long)n * P;
+  return dim == 3 ? (long long)n * P * (conv3_ok(dim, P) ? n : P) : (long long)n * P;
 }
 
-int conv_kernels_per_pass(int dim) { return dim == 3 ? 5 : 3; }
+int conv_kernels_per_pass(int dim, int P) { return dim == 3 && !conv3_ok(dim, P) ? 5 : 3; }
 
 // x rows of a field: row q (q < nrows) holds pixels q*n .. q*n + n - 1 and
 // its transform is row  tx * tstride + (q / n) * slab + (q % n) * P  of R.
@@ -445,23 +447,7 @@ __global__ void __launch_bounds__(256) conv_rows_inv(const ConvOp op, const floa
         }
         op.out[idx] = y;
         if (op.out2) op.out2[idx] = y;
-        if constexpr (DK == DOTS_RV) {
-          acc[0] = c_add(acc[0], c_cjmul(aux, y));
-        } else if constexpr (DK == DOTS_TS) {
-          acc[1] = c_add(acc[1], c_cjmul(y, src));
-          acc[2].x = fmaf(y.x, y.x, fmaf(y.y, y.y, acc[2].x));
-        } else if constexpr (DK == DOTS_RES) {
-          acc[0].x = fmaf(aux.x, aux.x, fmaf(aux.y, aux.y, acc[0].x));
-          acc[2].x = fmaf(y.x, y.x, fmaf(y.y, y.y, acc[2].x));
-        } else if constexpr (DK == DOTS_ANY) {
-#pragma unroll
-          for (int s = 0; s < DOT_SLOTS; ++s) {
-            if (op.dot_a[s]) {
-              const float2 a = pick(op.dot_a[s], y, src, aux), b = pick(op.dot_b[s], y, src, aux);
-              acc[s] = c_add(acc[s], c_cjmul(a, b));
-            }
-          }
-        }
+        dots_accumulate<DK>(op, acc, y, src, aux);
       }
   }
   if constexpr (DK != DOTS_NONE)
@@ -474,7 +460,7 @@ static void launch_cols(cisor_ctx* c, const ConvOp& op, int nslab, long long es,
   constexpr size_t SMB = ColSmem<P, MODE, NT>::BYTES;
   const ColGeo geo{c->n, P / W, es, slab, c->rtstride, op.tx_div, op.tx0};
   dim3 g((P / W) * nslab, op.ntx);
-  if constexpr (P <= 256) {  // 3D grids use P <= 256
+  if constexpr (P == 256) {  // 3D grids with smaller P take conv3d.cu
     if (c->dim == 3) {
       (void)launch_pdl(conv_cols<P, MODE, ADJ, NT, true>, g, dim3(NT), SMB, c->stream, op.active, c->twst, c->ghat, c->R,
                        geo);
@@ -496,7 +482,7 @@ static cudaError_t cols_attr() {
 template <int P, bool ADJ, int NT>
 static cudaError_t cols_attrs() {
   cudaError_t e = cols_attr<P, COL_G, ADJ, NT, false>();
-  if constexpr (P <= 256) {
+  if constexpr (P == 256) {
     if (e == cudaSuccess) e = cols_attr<P, COL_G, ADJ, NT, true>();
     if (e == cudaSuccess) e = cols_attr<P, COL_FWD, ADJ, NT, true>();
     if (e == cudaSuccess) e = cols_attr<P, COL_INV, ADJ, NT, true>();
@@ -510,7 +496,7 @@ static cisor_status conv_init_t() {
     for (int adj = 0; adj < 2; ++adj) {
       CISOR_CUDA(cudaFuncSetAttribute(adj ? conv_cols_2s<P, COL_G, true, false> : conv_cols_2s<P, COL_G, false, false>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smb));
-      if constexpr (P <= 256) {
+      if constexpr (P == 256) {
         CISOR_CUDA(cudaFuncSetAttribute(adj ? conv_cols_2s<P, COL_G, true, true> : conv_cols_2s<P, COL_G, false, true>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smb));
         CISOR_CUDA(cudaFuncSetAttribute(adj ? conv_cols_2s<P, COL_FWD, true, true> : conv_cols_2s<P, COL_FWD, false, true>,
@@ -535,7 +521,7 @@ static void launch_cols_2s(cisor_ctx* c, const ConvOp& op, int nslab, long long 
     typedef TwoStage<P> TS;
     const ColGeo geo{c->n, P / TS::W, es, slab, c->rtstride, op.tx_div, op.tx0};
     const dim3 g((P / TS::W) * nslab, op.ntx);
-    if constexpr (P <= 256) {
+    if constexpr (P == 256) {
       if (c->dim == 3) {
         (void)launch_pdl(conv_cols_2s<P, MODE, ADJ, true>, g, dim3(256), TS::SMEM, c->stream, op.active, c->tw, c->ghat,
                          c->R, geo);
@@ -573,6 +559,9 @@ static void cols_pass(cisor_ctx* c, const ConvOp& op, int nslab, long long es, l
 template <int P>
 static cisor_status conv_chunk_t(cisor_ctx* c, const ConvOp& op) {
   typedef ConvCfg<P> C;
+  if constexpr (P <= 128) {
+    if (c->dim == 3) return conv3_pass(c, op);
+  }
   if constexpr (P == 512) {  // the one-kernel cluster pass where the shape asks for it and the combination exists
     if (c->cols_nt == COLS_CLUSTER && conv_fused_ok(c)) {
       cudaError_t e = cudaSuccess;
@@ -594,16 +583,19 @@ static cisor_status conv_chunk_t(cisor_ctx* c, const ConvOp& op) {
     default: (void)launch_pdl(conv_rows_fwd<P, PRO_AXPY>, grow, dim3(256), 0, c->stream, op, c->twst, c->R, rg); break;
   }
   CISOR_CUDA(cudaGetLastError());
-  if (c->dim == 3) {
-    const long long PP = (long long)P * P;
-    cols_pass<P, COL_FWD>(c, op, n, P, PP);   // y, in each of the n z slabs
-    CISOR_CUDA(cudaGetLastError());
-    cols_pass<P, COL_G>(c, op, P, PP, P);     // z, for each of the P y frequencies
-    CISOR_CUDA(cudaGetLastError());
-    cols_pass<P, COL_INV>(c, op, n, P, PP);   // y back, n rows kept
-  } else {
-    cols_pass<P, COL_G>(c, op, 1, P, 0);
+  bool slabs = false;
+  if constexpr (P == 256) {
+    slabs = c->dim == 3;
+    if (slabs) {
+      const long long PP = (long long)P * P;
+      cols_pass<P, COL_FWD>(c, op, n, P, PP);   // y, in each of the n z slabs
+      CISOR_CUDA(cudaGetLastError());
+      cols_pass<P, COL_G>(c, op, P, PP, P);     // z, for each of the P y frequencies
+      CISOR_CUDA(cudaGetLastError());
+      cols_pass<P, COL_INV>(c, op, n, P, PP);   // y back, n rows kept
+    }
   }
+  if (!slabs) cols_pass<P, COL_G>(c, op, 1, P, 0);
   CISOR_CUDA(cudaGetLastError());
   const int dk = dots_kind(op);
 #define CISOR_ROWS_INV(E, D) \
@@ -626,7 +618,7 @@ static cisor_status conv_chunk_t(cisor_ctx* c, const ConvOp& op) {
   }
 #undef CISOR_ROWS_INV
   CISOR_CUDA(cudaGetLastError());
-  c->launches += conv_kernels_per_pass(c->dim);
+  c->launches += conv_kernels_per_pass(c->dim, c->P);
   return CISOR_OK;
 }
 
@@ -649,6 +641,7 @@ static cisor_status conv_pass_t(cisor_ctx* c, const ConvOp& op) {
 
 cisor_status conv_init(int P) {
   if (P == 512) CISOR_TRY(conv_fused_init());
+  if (P <= 128) CISOR_TRY(conv3_init(P));
   switch (P) {
     case 64: return conv_init_t<64>();
     case 128: return conv_init_t<128>();

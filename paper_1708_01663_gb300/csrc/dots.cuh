@@ -31,6 +31,26 @@ __device__ __forceinline__ float2 pick(int code, float2 y, float2 s, float2 a) {
   return code == OP_Y ? y : (code == OP_SRC ? s : a);
 }
 
+// adds one element's products of the set DK (y the result, src and aux the epilogue's other operands)
+template <int DK>
+__device__ __forceinline__ void dots_accumulate(const ConvOp& op, float2 acc[DOT_SLOTS], float2 y, float2 src,
+                                                float2 aux) {
+  if constexpr (DK == DOTS_RV) {
+    acc[0] = c_add(acc[0], c_cjmul(aux, y));
+  } else if constexpr (DK == DOTS_TS) {
+    acc[1] = c_add(acc[1], c_cjmul(y, src));
+    acc[2].x = fmaf(y.x, y.x, fmaf(y.y, y.y, acc[2].x));
+  } else if constexpr (DK == DOTS_RES) {
+    acc[0].x = fmaf(aux.x, aux.x, fmaf(aux.y, aux.y, acc[0].x));
+    acc[2].x = fmaf(y.x, y.x, fmaf(y.y, y.y, acc[2].x));
+  } else if constexpr (DK == DOTS_ANY) {
+#pragma unroll
+    for (int s = 0; s < DOT_SLOTS; ++s)
+      if (op.dot_a[s])
+        acc[s] = c_add(acc[s], c_cjmul(pick(op.dot_a[s], y, src, aux), pick(op.dot_b[s], y, src, aux)));
+  }
+}
+
 // Block-wide sum of three complex FP32 partials: warp shuffles, then the
 // per-warp sums pairwise in shared memory (all FP32), written to part.  Only
 // the slots in MASK (bit s: slot s) are reduced; the others are written as 0.

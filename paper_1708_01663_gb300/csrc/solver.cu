@@ -265,7 +265,7 @@ static cisor_status residual_pass(cisor_ctx* c, int adjoint, const float2* b, co
 
 // x += alpha p + omega s ; r = s - omega t ; <rhat, r>, <r, r>, then rho', beta, convergence
 static cisor_status update_step(cisor_ctx* c, float2* x, int ntx) {
-  const int RB = conv_rows_per_block(c->P);
+  const int RB = conv_rows_per_block(c->dim, c->P);
   dim3 g(c->nblk * c->ncomp, ntx);
   (void)launch_pdl(bicg_update_kernel, g, dim3(256), 0, c->stream, c->n, c->nrows * c->ncomp, RB, c->nblk * c->ncomp,
                    (const int*)c->active, (const double*)c->scal, x, (const float2*)c->p, (const float2*)c->s,

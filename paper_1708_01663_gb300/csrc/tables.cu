@@ -330,6 +330,7 @@ cisor_status build_tables(cisor_ctx* c) {
     case 512: CISOR_TRY(spectrum_fft<512>(c, cbuf, tw64)); CISOR_TRY(stage_twiddles<512>(c)); break;
     default: set_error("unsupported FFT size %d", P); return CISOR_ERR_INVALID_ARG;
   }
+  if (conv3_ok(d, P)) CISOR_TRY(conv3_tables(c));
   long long MN = (long long)c->M * c->N;
   long long TN = (long long)c->T * c->N;
   if (c->ncomp == 3) {  // vectorial model: dyadic sensing row and polarised plane waves

@@ -125,7 +125,7 @@ static VecEpiArgs stencil_args(cisor_ctx* c) {
   VecEpiArgs a{};
   a.n = c->n;
   a.N = c->N;
-  a.RB = conv_rows_per_block(c->P);
+  a.RB = conv_rows_per_block(c->dim, c->P);
   a.nblk = c->nblk;
   a.part = c->part;
   a.inv_k2 = (float)(1.0 / (c->k * c->k));
