@@ -104,7 +104,7 @@ static cisor_status data_core(cisor_ctx* c, const cisor_solve_opts* o, double* D
   if (o->x0_mode != 2 || !c->have_u) CISOR_CUDA(cudaMemcpyAsync(c->u, c->u_in, vb, cudaMemcpyDeviceToDevice, c->stream));
   int nb1 = 0;
   c->have_w = 0;
-  cisor_status s1 = solve_batch(c, 0, c->f, c->u_in, c->u, c->T, o->tol, o->max_iter, &li->iters_max, &li->iters_mean,
+  cisor_status s1 = solve_batch(c, 0, c->f, c->u_in, c->u, 0, c->T, o->tol, o->max_iter, &li->iters_max, &li->iters_mean,
                                 &li->resid_max, &nb1);
   if (!solve_ok(s1)) return s1;
   c->have_u = 1;
@@ -123,28 +123,15 @@ static cisor_status adjoint_core(cisor_ctx* c, const cisor_solve_opts* o, double
                                  float2* zstep, cisor_solve_info* li) {
   const size_t vb = sizeof(float2) * (size_t)c->T * c->Nf;
   CISOR_TRY(sense_adjoint(c, c->f, c->w, c->z, c->b, c->T));
-  if (o->x0_mode != 2 || !c->have_v) CISOR_CUDA(cudaMemsetAsync(c->vadj, 0, vb, c->stream));
+  const int cold = o->x0_mode != 2 || !c->have_v;
+  if (cold) CISOR_CUDA(cudaMemsetAsync(c->vadj, 0, vb, c->stream));
   int nb2 = 0;
-  cisor_status s2 = solve_batch(c, 1, c->f, c->b, c->vadj, c->T, o->tol, o->max_iter, &li->adj_iters_max,
+  cisor_status s2 = solve_batch(c, 1, c->f, c->b, c->vadj, cold, c->T, o->tol, o->max_iter, &li->adj_iters_max,
                                 &li->adj_iters_mean, &li->adj_resid_max, &nb2);
   if (!solve_ok(s2)) return s2;
   c->have_v = 1;
   li->n_not_converged += nb2;
-  if (c->ncomp == 3) {
-    CISOR_TRY(vec_gz(c));  // z + conv_{G^H}(v + D v / k^2)
-  } else {
-    ConvOp op{};
-    op.adjoint = 1;
-    op.mul_f = 0;
-    op.prologue = PRO_COPY;
-    op.src = c->vadj;
-    op.epilogue = EPI_CONV_ADD;
-    op.aux = c->z;
-    op.out = c->gz;
-    op.f = c->f;
-    op.ntx = c->T;
-    CISOR_TRY(conv_pass(c, op));
-  }
+  CISOR_TRY(adjoint_fields(c));
   CISOR_TRY(grad_assemble(c, c->u, c->gz, s, gamma, c->grad, zstep, c->T));
   return s2;
 }
@@ -520,7 +507,7 @@ cisor_status cisor_forward(cisor_ctx* c, const void* f, const void* u_in, const 
   }
   cisor_solve_info li{};
   int nb = 0;
-  cisor_status st = solve_batch(c, 0, c->f, b, c->u, c->T, o->tol, o->max_iter, &li.iters_max, &li.iters_mean,
+  cisor_status st = solve_batch(c, 0, c->f, b, c->u, 0, c->T, o->tol, o->max_iter, &li.iters_max, &li.iters_mean,
                                 &li.resid_max, &nb);
   if (!solve_ok(st)) return st;
   li.n_not_converged = nb;

@@ -210,7 +210,7 @@ cisor_status cisor_batch_forward(cisor_batch* b, const void* const* f, void* con
     rhs[i] = c->u_in;
   }
   std::vector<SolveStat> st(np);
-  cisor_status s = solve_multi(b->ctx.data(), np, 0, rhs.data(), o->tol, o->max_iter, b->ms, st.data());
+  cisor_status s = solve_multi(b->ctx.data(), np, 0, rhs.data(), nullptr, o->tol, o->max_iter, b->ms, st.data());
   if (!solve_ok(s)) return s;
   bool host_out = false;
   for (int i = 0; i < np; ++i) {
@@ -253,7 +253,8 @@ cisor_status cisor_batch_grad(cisor_batch* b, const void* const* f, const void* 
     rhs[i] = c->u_in;
   }
   std::vector<SolveStat> fw(np), ad(np);
-  cisor_status s1 = solve_multi(b->ctx.data(), np, 0, rhs.data(), o->tol, o->max_iter, b->ms, fw.data());
+  std::vector<int> cold(np);
+  cisor_status s1 = solve_multi(b->ctx.data(), np, 0, rhs.data(), nullptr, o->tol, o->max_iter, b->ms, fw.data());
   if (!solve_ok(s1)) return s1;
   for (int i = 0; i < np; ++i) {
     cisor_ctx* c = b->ctx[i];
@@ -261,26 +262,17 @@ cisor_status cisor_batch_grad(cisor_batch* b, const void* const* f, const void* 
     c->have_u = 1;
     CISOR_TRY(residual_and_D(c, c->f, c->u, c->yobs, c->Y, c->w, c->T));
     CISOR_TRY(sense_adjoint(c, c->f, c->w, c->z, c->b, c->T));
-    if (o->x0_mode == 0 || !c->have_v) CISOR_CUDA(cudaMemsetAsync(c->vadj, 0, vb, c->stream));
+    cold[i] = o->x0_mode == 0 || !c->have_v;
+    if (cold[i]) CISOR_CUDA(cudaMemsetAsync(c->vadj, 0, vb, c->stream));
     rhs[i] = c->b;
   }
-  cisor_status s2 = solve_multi(b->ctx.data(), np, 1, rhs.data(), o->tol, o->max_iter, b->ms, ad.data());
+  cisor_status s2 = solve_multi(b->ctx.data(), np, 1, rhs.data(), cold.data(), o->tol, o->max_iter, b->ms, ad.data());
   if (!solve_ok(s2)) return s2;
   bool host_out = false;
   for (int i = 0; i < np; ++i) {
     cisor_ctx* c = b->ctx[i];
     c->have_v = 1;
-    ConvOp op{};
-    op.adjoint = 1;
-    op.mul_f = 0;
-    op.prologue = PRO_COPY;
-    op.src = c->vadj;
-    op.epilogue = EPI_CONV_ADD;
-    op.aux = c->z;
-    op.out = c->gz;
-    op.f = c->f;
-    op.ntx = c->T;
-    CISOR_TRY(conv_pass(c, op));
+    CISOR_TRY(adjoint_fields(c));
     CISOR_TRY(grad_assemble(c, c->u, c->gz, nullptr, 0.0, c->grad, nullptr, c->T));
     host_out |= is_host(grad_out[i]);
     CISOR_CUDA(cudaMemcpyAsync(grad_out[i], c->grad, sizeof(float2) * c->N, cudaMemcpyDefault, c->stream));

@@ -117,6 +117,7 @@ struct cisor_ctx {
   int have_w;          // 1 from cisor_data_term until an entry point overwrites the u or w it left
   float2* f_ck;        // [N] the point of the last cisor_data_term (its backward half's f)
   float2 *z, *gz;     // H^H w and z + G^H v
+  int gz_ready;       // the last adjoint solve's final residual pass left gz
   float2 *f, *fz, *grad, *work_n;  // [N]
   float2 *Y, *w, *yobs;          // [T, M]
   unsigned char* rx_mask;        // [T, M] active receivers (NULL: all), set by cisor_set_rx_mask
@@ -206,6 +207,8 @@ struct ConvOp {
   const float2* aux;      // epilogue auxiliary vector (rhat, b, z)
   float2* out;            // epilogue output
   float2* out2;           // second epilogue output (copy of out), may be null
+  float2* gz;             // EPI_RESID: also gz = zadd + the bare convolution (before the f factor); may be null
+  const float2* zadd;
   int dot_a[DOT_SLOTS], dot_b[DOT_SLOTS];  // operand codes per dot slot
   const int* active;      // may be null
   const double* scal;     // per-transmitter scalars (alpha, beta, omega)
@@ -274,7 +277,9 @@ cisor_status conv3_tables(cisor_ctx* c);   // c->gplane from c->ghat
 cisor_status conv3_pass(cisor_ctx* c, const ConvOp& op);
 
 // solver.cu
-cisor_status solve_batch(cisor_ctx* c, int adjoint, const float2* f, const float2* b, float2* x,
+// Solves A x = b (adjoint = 0) or A^H x = b (1) from the x given; x_zero: x is zero.  An adjoint solve also leaves
+// gz = c->z + G^H x (Prop. 1) in c->gz and sets c->gz_ready whenever it recomputed the true residual.
+cisor_status solve_batch(cisor_ctx* c, int adjoint, const float2* f, const float2* b, float2* x, int x_zero,
                          int ntx, double tol, int max_iter, int* iters_max, double* iters_mean,
                          double* resid_max, int* n_bad);
 
@@ -296,8 +301,9 @@ struct MultiSolve {
   int* h_loop_count;            // pinned
   int use_while;
 };
-cisor_status solve_multi(cisor_ctx* const* cs, int np, int adjoint, const float2* const* b, double tol, int max_iter,
-                         MultiSolve& ms, SolveStat* st);
+cisor_status solve_multi(cisor_ctx* const* cs, int np, int adjoint, const float2* const* b, const int* x_zero,
+                         double tol, int max_iter, MultiSolve& ms, SolveStat* st);
+cisor_status adjoint_fields(cisor_ctx* c);  // c->gz = c->z + G^H c->vadj unless the adjoint solve left it
 
 // vector.cu: the vectorial model (appendix).  Matvec over [ntx, 3, N] fields:
 // A x = x - C - D C / k^2 (C = conv_G(f x)) or A^H x = x - conj(f) conv_{G^H}(x + D x / k^2),
@@ -309,6 +315,8 @@ struct VecOp {
   const float2* aux;      // b of EPI_RESID, dot operand
   float2* out;
   float2* out2;
+  float2* gz;             // as in ConvOp (adjoint only)
+  const float2* zadd;
   int dot_a[DOT_SLOTS], dot_b[DOT_SLOTS];
   const int* active;
   int ntx;

@@ -435,6 +435,7 @@ __global__ void __launch_bounds__(256) conv_rows_inv(const ConvOp op, const floa
         const long long pix = (long long)iy * n + ix;
         const long long idx = tx * N + pix;
         float2 c = v[q * RL + r];
+        if (EPI == EPI_RESID && op.gz) op.gz[idx] = c_add(c, op.zadd[idx]);
         if (postf) c = c_cjmul(op.f[pix], c);
         const float2 src = pre_src[q * RL + r], aux = pre_aux[q * RL + r];
         float2 y;

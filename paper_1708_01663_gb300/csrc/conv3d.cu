@@ -342,6 +342,7 @@ __global__ void __launch_bounds__(256) conv3_rows_inv(const ConvOp op, const flo
     if (!rowok || ix >= n) continue;
     const long long idx = base + ix;
     float2 c = v[k];
+    if (EPI == EPI_RESID && op.gz) op.gz[idx] = c_add(c, op.zadd[idx]);
     if (postf) c = c_cjmul(op.f[row0 + ix], c);
     const float2 src = pre_src[k], aux = pre_aux[k];
     float2 y;

@@ -218,6 +218,7 @@ __global__ void __launch_bounds__(ZNT, 1) conv_fused512(const ConvOp op, const f
             const long long pix = (long long)iy * n + ix;
             const long long idx = tx * N + pix;
             float2 cv = v[q * RL + r];
+            if (EPI == EPI_RESID && op.gz) op.gz[idx] = c_add(cv, op.zadd[idx]);
             if (postf) cv = c_cjmul(op.f[pix], cv);
             const float2 src = pre_src[q * RL + r], aux = pre_aux[q * RL + r];
             float2 y;

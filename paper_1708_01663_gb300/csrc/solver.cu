@@ -24,6 +24,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "dots.cuh"
 
 namespace cisor {
 
@@ -212,6 +213,26 @@ __global__ void __launch_bounds__(256) bicg_update_kernel(int n, int nrows, int 
   }
 }
 
+// r = rhat = b for a solve that starts from x = 0 (A 0 = 0 needs no pass); partials <b, b> in slots 0 and 2.  The
+// same rows per CTA as bicg_update_kernel.
+__global__ void __launch_bounds__(256) bicg_zero_start_kernel(int n, int nrows, int RB, int nblk,
+                                                              const float2* __restrict__ b, float2* __restrict__ r,
+                                                              float2* __restrict__ rhat, float* __restrict__ part) {
+  pdl_trigger();
+  pdl_wait();
+  const int t = blockIdx.y, row0 = blockIdx.x * RB, cnt = min(RB, nrows - row0) * n;
+  const long long base = ((long long)t * nrows + row0) * n;
+  float2 acc[DOT_SLOTS] = {};
+  for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+    const float2 v = b[base + e];
+    r[base + e] = v;
+    rhat[base + e] = v;
+    acc[0].x = fmaf(v.x, v.x, fmaf(v.y, v.y, acc[0].x));
+  }
+  acc[2] = acc[0];
+  block_dots<256, 5>(acc, reinterpret_cast<float2*>(part) + ((size_t)t * nblk + blockIdx.x) * DOT_SLOTS);
+}
+
 static cisor_status scalar_step(cisor_ctx* c, int mode, int ntx) {
   (void)launch_pdl(bicg_scalar_kernel, dim3(ntx), dim3(32), 0, c->stream, mode, c->nblk * c->ncomp,
                    (const float*)c->part, c->scal, c->active, c->iters, c->txflag, (const double*)c->sparams);
@@ -231,8 +252,9 @@ static ConvOp base_op(cisor_ctx* c, int adjoint, int ntx) {
   return op;
 }
 
-// r = b - A x ; rhat = r ; partials <b,b> (slot 0) and <r,r> (slot 2)
-static cisor_status residual_pass(cisor_ctx* c, int adjoint, const float2* b, const float2* x, int ntx) {
+// r = b - A x ; rhat = r ; partials <b,b> (slot 0) and <r,r> (slot 2).  b - A^H x = b - x + conj(f) G^H x holds the
+// G^H v that the gradient needs of the solution, so the final pass of an adjoint solve (gz) stores z + G^H x too.
+static cisor_status residual_pass(cisor_ctx* c, int adjoint, const float2* b, const float2* x, int ntx, bool gz) {
   if (c->ncomp == 3) {
     VecOp vo{};
     vo.adjoint = adjoint;
@@ -241,6 +263,8 @@ static cisor_status residual_pass(cisor_ctx* c, int adjoint, const float2* b, co
     vo.aux = b;
     vo.out = c->r;
     vo.out2 = c->rhat;
+    vo.gz = gz ? c->gz : nullptr;
+    vo.zadd = c->z;
     vo.dot_a[0] = OP_AUX;
     vo.dot_b[0] = OP_AUX;
     vo.dot_a[2] = OP_Y;
@@ -256,6 +280,8 @@ static cisor_status residual_pass(cisor_ctx* c, int adjoint, const float2* b, co
   op.aux = b;
   op.out = c->r;
   op.out2 = c->rhat;
+  op.gz = gz ? c->gz : nullptr;
+  op.zadd = c->z;
   op.dot_a[0] = OP_AUX;
   op.dot_b[0] = OP_AUX;
   op.dot_a[2] = OP_Y;
@@ -342,6 +368,23 @@ static cisor_status enqueue_iteration(cisor_ctx* c, int adjoint, float2* x, int 
   CISOR_TRY(conv_pass(c, op2));
   CISOR_TRY(scalar_step(c, SCM_OMEGA, ntx));
   return update_step(c, x, ntx);
+}
+
+cisor_status adjoint_fields(cisor_ctx* c) {
+  if (c->gz_ready) return CISOR_OK;
+  c->gz_ready = 1;
+  if (c->ncomp == 3) return vec_gz(c);  // z + conv_{G^H}(v + D v / k^2)
+  ConvOp op{};
+  op.adjoint = 1;
+  op.mul_f = 0;
+  op.prologue = PRO_COPY;
+  op.src = c->vadj;
+  op.epilogue = EPI_CONV_ADD;
+  op.aux = c->z;
+  op.out = c->gz;
+  op.f = c->f;
+  op.ntx = c->T;
+  return conv_pass(c, op);
 }
 
 static cisor_status get_graph(cisor_ctx* c, int adjoint, float2* x, int ntx, cudaGraphExec_t* out) {
@@ -493,8 +536,8 @@ static cisor_status read_active(cisor_ctx* c, int ntx, int* n_active) {
 
 // Sets the solve parameters, zeroes p and v, forms r = b - A x0, rhat = r and
 // runs the INIT scalar step (all on c->stream).
-static cisor_status init_solve(cisor_ctx* c, int adjoint, const float2* b, float2* x, int ntx, double tol,
-                               int max_iter) {
+static cisor_status init_solve(cisor_ctx* c, int adjoint, const float2* b, float2* x, int x_zero, int ntx,
+                               double tol, int max_iter) {
   const size_t vb = sizeof(float2) * (size_t)ntx * c->Nf;
   // pageable source: the copy is staged before cudaMemcpyAsync returns, so the stack array may go
   const double hp[2] = {tol, (double)max_iter};
@@ -502,13 +545,22 @@ static cisor_status init_solve(cisor_ctx* c, int adjoint, const float2* b, float
   CISOR_CUDA(cudaMemsetAsync(c->p, 0, vb, c->stream));
   CISOR_CUDA(cudaMemsetAsync(c->v, 0, vb, c->stream));
   CISOR_CUDA(cudaMemsetAsync(c->active, 0, sizeof(int) * ntx, c->stream));
-  CISOR_TRY(residual_pass(c, adjoint, b, x, ntx));
+  if (adjoint) c->gz_ready = 0;
+  if (x_zero) {
+    CISOR_CUDA(launch_pdl(bicg_zero_start_kernel, dim3(c->nblk * c->ncomp, ntx), dim3(256), 0, c->stream, c->n,
+                          c->nrows * c->ncomp, conv_rows_per_block(c->dim, c->P), c->nblk * c->ncomp, b, c->r,
+                          c->rhat, c->part));
+    c->launches += 1;
+  } else {
+    CISOR_TRY(residual_pass(c, adjoint, b, x, ntx, false));
+  }
   return scalar_step(c, SCM_INIT, ntx);
 }
 
 // True residual r = b - A x and the restart decision (SCM_TRUE).
 static cisor_status true_residual(cisor_ctx* c, int adjoint, const float2* b, float2* x, int ntx) {
-  CISOR_TRY(residual_pass(c, adjoint, b, x, ntx));
+  CISOR_TRY(residual_pass(c, adjoint, b, x, ntx, adjoint != 0));
+  if (adjoint) c->gz_ready = 1;
   return scalar_step(c, SCM_TRUE, ntx);
 }
 
@@ -546,10 +598,11 @@ static cisor_status collect_stats(cisor_ctx* c, int adjoint, int ntx, double tol
   return CISOR_OK;
 }
 
-cisor_status solve_batch(cisor_ctx* c, int adjoint, const float2* f, const float2* b, float2* x, int ntx, double tol,
-                         int max_iter, int* iters_max, double* iters_mean, double* resid_max, int* n_bad) {
+cisor_status solve_batch(cisor_ctx* c, int adjoint, const float2* f, const float2* b, float2* x, int x_zero, int ntx,
+                         double tol, int max_iter, int* iters_max, double* iters_mean, double* resid_max,
+                         int* n_bad) {
   (void)f;  // the operator always reads the context's copy of f (c->f), baked into the graphs
-  CISOR_TRY(init_solve(c, adjoint, b, x, ntx, tol, max_iter));
+  CISOR_TRY(init_solve(c, adjoint, b, x, x_zero, ntx, tol, max_iter));
   int nact = 0;
   CISOR_TRY(read_active(c, ntx, &nact));
   cudaGraphExec_t ge = nullptr;
@@ -583,10 +636,11 @@ cisor_status solve_batch(cisor_ctx* c, int adjoint, const float2* f, const float
 // fork from ms.main to every context's stream, each context's chunk of
 // iterations on its own stream, join back.  One cudaGraphLaunch advances all
 // problems; converged transmitters and finished problems exit their CTAs at once.
-cisor_status solve_multi(cisor_ctx* const* cs, int np, int adjoint, const float2* const* b, double tol, int max_iter,
-                         MultiSolve& ms, SolveStat* st) {
+cisor_status solve_multi(cisor_ctx* const* cs, int np, int adjoint, const float2* const* b, const int* x_zero,
+                         double tol, int max_iter, MultiSolve& ms, SolveStat* st) {
   auto xof = [&](cisor_ctx* c) { return adjoint ? c->vadj : c->u; };
-  for (int i = 0; i < np; ++i) CISOR_TRY(init_solve(cs[i], adjoint, b[i], xof(cs[i]), cs[i]->T, tol, max_iter));
+  for (int i = 0; i < np; ++i)
+    CISOR_TRY(init_solve(cs[i], adjoint, b[i], xof(cs[i]), x_zero ? x_zero[i] : 0, cs[i]->T, tol, max_iter));
   auto count = [&](int* total) -> cisor_status {
     for (int i = 0; i < np; ++i)
       CISOR_CUDA(cudaMemcpyAsync(cs[i]->h_active, cs[i]->active, sizeof(int) * cs[i]->T, cudaMemcpyDeviceToHost,

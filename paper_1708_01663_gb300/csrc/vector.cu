@@ -184,6 +184,8 @@ cisor_status vec_matvec(cisor_ctx* c, const VecOp& op) {
   co.aux = op.aux;
   co.out = op.out;
   co.out2 = op.out2;
+  co.gz = op.gz;
+  co.zadd = op.zadd;
   for (int s = 0; s < DOT_SLOTS; ++s) {
     co.dot_a[s] = op.dot_a[s];
     co.dot_b[s] = op.dot_b[s];
