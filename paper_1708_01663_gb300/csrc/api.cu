@@ -38,6 +38,22 @@ static bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Whether kernels on c's stream can use p in place: memory of c's device, aligned for complex64.  Anything else
+// (host, managed, another device's, odd addresses) goes through the context's buffers.
+static bool in_place(const cisor_ctx* c, const void* p) {
+  cudaPointerAttributes a;
+  if (!p || ((uintptr_t)p & 7)) return false;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == c->device;
+}
+static bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+  return a && b && x < y + nb && y < x + na;
+}
+
 __global__ void scale_copy_kernel(const float2* __restrict__ in, float2* __restrict__ out, long long n, float s) {
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = make_float2(in[i].x * s, in[i].y * s);
@@ -63,6 +79,13 @@ struct Call {
     if (!is_device_ptr(dst)) host_out = true;
     CISOR_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, c->stream));
     return CISOR_OK;
+  }
+  // *use: an input where kernels can read it: src itself, or its copy in buf.  out, out2: what they write meanwhile.
+  cisor_status operand(const float2** use, const void* src, float2* buf, size_t bytes, const void* out = nullptr,
+                       size_t out_bytes = 0, const void* out2 = nullptr) {
+    const bool direct = in_place(c, src) && !overlap(src, bytes, out, out_bytes) && !overlap(src, bytes, out2, out_bytes);
+    *use = direct ? (const float2*)src : buf;
+    return direct ? CISOR_OK : in(buf, src, bytes);
   }
   cisor_status leave() {
     CISOR_CUDA(cudaEventRecord(c->ev_b, c->stream));
@@ -98,8 +121,9 @@ static bool solve_ok(cisor_status s) {
 
 // Forward half of the gradient machinery on c->f (the point) and c->yobs
 // (the data): forward solve into c->u (kept: the fields are the checkpoint the
-// backward half needs), Z, w = Z - y and D.
-static cisor_status data_core(cisor_ctx* c, const cisor_solve_opts* o, double* D, cisor_solve_info* li) {
+// backward half needs), Z, w = Z - y and D, which is in c->h_dsum[0] once the
+// caller has waited for the stream.
+static cisor_status data_core(cisor_ctx* c, const cisor_solve_opts* o, cisor_solve_info* li) {
   const size_t vb = sizeof(float2) * (size_t)c->T * c->Nf;
   if (o->x0_mode != 2 || !c->have_u) CISOR_CUDA(cudaMemcpyAsync(c->u, c->u_in, vb, cudaMemcpyDeviceToDevice, c->stream));
   int nb1 = 0;
@@ -111,8 +135,6 @@ static cisor_status data_core(cisor_ctx* c, const cisor_solve_opts* o, double* D
   li->n_not_converged = nb1;
   CISOR_TRY(residual_and_D(c, c->f, c->u, c->yobs, c->Y, c->w, c->T));
   CISOR_CUDA(cudaMemcpyAsync(c->h_dsum, c->dsum, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  CISOR_CUDA(cudaStreamSynchronize(c->stream));
-  if (D) *D = c->h_dsum[0];
   return s1;
 }
 
@@ -146,10 +168,11 @@ static void drop_data_term(cisor_ctx* c) { c->have_w = 0; }
 static cisor_status grad_core(cisor_ctx* c, const cisor_solve_opts* o, double gamma, const float2* s, float2* zstep,
                               double* D, cisor_solve_info* info) {
   cisor_solve_info li{};
-  cisor_status s1 = data_core(c, o, D, &li);
+  cisor_status s1 = data_core(c, o, &li);
   if (!solve_ok(s1)) return s1;
   cisor_status s2 = adjoint_core(c, o, gamma, s, zstep, &li);
   if (!solve_ok(s2)) return s2;
+  *D = c->h_dsum[0];  // the adjoint solve waited for the stream after D was copied out
   if (info) *info = li;
   return worse(s1, s2);
 }
@@ -181,7 +204,7 @@ static void free_ctx(cisor_ctx* c) {
                  c->tv_r0, c->tv_r1, c->tv_p, c->rx_mask, c->tva0, c->tva1, c->vbuf, c->f_ck, c->Ht};
   for (void* p : dev)
     if (p) cudaFree(p);
-  if (c->h_active) cudaFreeHost(c->h_active);
+  if (c->h_stat) cudaFreeHost(c->h_stat);
   if (c->h_dsum) cudaFreeHost(c->h_dsum);
   if (c->h_tc_err) cudaFreeHost(c->h_tc_err);
   if (c->ev_a) cudaEventDestroy(c->ev_a);
@@ -189,6 +212,14 @@ static void free_ctx(cisor_ctx* c) {
   if (c->stream) cudaStreamDestroy(c->stream);
   delete c;
 }
+
+static bool two_stage_ok(const cisor_ctx* c) { return c->P == 128 || c->P == 256 || (c->dim == 2 && c->P == 512); }
+
+// Column shape of a context until it is set or autotuned, from back-to-back passes on 1 to 64 transmitters.  P = 512
+// and 256: two-stage (64 transmitters 90 against 107 and 126 us with 512 and 256 threads; P = 256: 23 against 28 us;
+// one transmitter: 12 against 13 us).  P <= 128: 256 threads, whose smaller CTAs suit the few columns there are (P =
+// 128, 8 transmitters: 7.9 against 9.1 us with 512 threads, 64 of them: 12.8 against 13.2; P = 64: 6.3 against 7.0).
+static int default_shape(const cisor_ctx* c) { return c->P >= 256 && two_stage_ok(c) ? COLS_TWO_STAGE : 256; }
 
 }  // namespace cisor
 
@@ -283,7 +314,7 @@ cisor_status cisor_create(cisor_ctx** out, const cisor_geometry* g, void* stream
   c->user_stream = (cudaStream_t)stream;
   c->graph_chunk = 4;
   c->use_while = 0;  // host-driven chunks by default: profilers list the kernels of these graphs
-  c->cols_nt = 512;
+  c->cols_nt = default_shape(c);
   conv_geometry(c);
   {
     // split-K of the forward sensing GEMM: about 4 CTAs per SM, chunks of >= 256 pixels
@@ -373,7 +404,8 @@ cisor_status cisor_create(cisor_ctx** out, const cisor_geometry* g, void* stream
   ALLOC(c->tva1, sizeof(float) * 2 * (2 * d + 1) * c->N);
 #undef ALLOC
   {
-    cudaError_t e = cudaMallocHost((void**)&c->h_active, sizeof(int) * c->T);
+    cudaError_t e = cudaHostAlloc((void**)&c->h_stat, sizeof(cisor_txstat) * c->T, cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&c->stat, c->h_stat, 0);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_dsum, sizeof(double) * 4);
     if (e != cudaSuccess) return fail(cuda_fail(e, "cudaMallocHost", __FILE__, __LINE__));
   }
@@ -441,11 +473,12 @@ cisor_status cisor_incident(cisor_ctx* c, void* out) {
 }
 
 // y = A x (or A^H x) for nvec fields, no dot products
-static cisor_status matvec_once(cisor_ctx* c, int adjoint, int nvec, const float2* x, float2* y) {
+static cisor_status matvec_once(cisor_ctx* c, int adjoint, int nvec, const float2* f, const float2* x, float2* y) {
   if (c->ncomp == 3) {
     VecOp vo{};
     vo.adjoint = adjoint ? 1 : 0;
     vo.epilogue = EPI_MATVEC;
+    vo.f = f;
     vo.x = x;
     vo.out = y;
     vo.ntx = nvec;
@@ -459,7 +492,7 @@ static cisor_status matvec_once(cisor_ctx* c, int adjoint, int nvec, const float
   op.epilogue = EPI_MATVEC;
   op.esrc = x;
   op.out = y;
-  op.f = c->f;
+  op.f = f;
   op.ntx = nvec;
   return conv_pass(c, op);
 }
@@ -472,10 +505,12 @@ cisor_status cisor_apply_A(cisor_ctx* c, const void* f, const void* x, void* y, 
   Call call(c);
   CISOR_TRY(call.enter());
   const size_t vb = sizeof(float2) * (size_t)nvec * c->Nf;
-  CISOR_TRY(call.in(c->f, f, sizeof(float2) * c->N));
-  CISOR_TRY(call.in(c->s, x, vb));
-  CISOR_TRY(matvec_once(c, adjoint, nvec, c->s, c->tv));
-  CISOR_TRY(call.out(y, c->tv, vb));
+  const float2 *fd, *xd;
+  CISOR_TRY(call.operand(&fd, f, c->f, sizeof(float2) * c->N, y, vb));
+  CISOR_TRY(call.operand(&xd, x, c->s, vb, y, vb));
+  const bool direct = in_place(c, y);
+  CISOR_TRY(matvec_once(c, adjoint, nvec, fd, xd, direct ? (float2*)y : c->tv));
+  if (!direct) CISOR_TRY(call.out(y, c->tv, vb));
   return call.leave();
 }
 
@@ -529,10 +564,12 @@ cisor_status cisor_sense(cisor_ctx* c, const void* f, const void* u, void* Z_out
   }
   Call call(c);
   CISOR_TRY(call.enter());
-  CISOR_TRY(call.in(c->f, f, sizeof(float2) * c->N));
-  CISOR_TRY(call.in(c->s, u, sizeof(float2) * (size_t)c->T * c->Nf));
-  CISOR_TRY(sense_forward(c, c->f, c->s, c->Y, c->T));
-  CISOR_TRY(call.out(Z_out, c->Y, sizeof(float2) * (size_t)c->T * c->M));
+  const float2 *fd, *ud;  // (the GEMM has read both before its reduction writes Z)
+  CISOR_TRY(call.operand(&fd, f, c->f, sizeof(float2) * c->N));
+  CISOR_TRY(call.operand(&ud, u, c->s, sizeof(float2) * (size_t)c->T * c->Nf));
+  const bool direct = in_place(c, Z_out);
+  CISOR_TRY(sense_forward(c, fd, ud, direct ? (float2*)Z_out : c->Y, c->T));
+  if (!direct) CISOR_TRY(call.out(Z_out, c->Y, sizeof(float2) * (size_t)c->T * c->M));
   return call.leave();
 }
 
@@ -544,12 +581,16 @@ cisor_status cisor_sense_adjoint(cisor_ctx* c, const void* f, const void* w, voi
   Call call(c);
   CISOR_TRY(call.enter());
   drop_data_term(c);  // c->w is overwritten
-  CISOR_TRY(call.in(c->f, f, sizeof(float2) * c->N));
-  CISOR_TRY(call.in(c->w, w, sizeof(float2) * (size_t)c->T * c->M));
-  CISOR_TRY(sense_adjoint(c, c->f, c->w, c->z, c->b, c->T));
   const size_t vb = sizeof(float2) * (size_t)c->T * c->Nf;
-  CISOR_TRY(call.out(z_out, c->z, vb));
-  CISOR_TRY(call.out(b_out, c->b, vb));
+  const float2 *fd, *wd;
+  CISOR_TRY(call.operand(&fd, f, c->f, sizeof(float2) * c->N, z_out, vb, b_out));
+  CISOR_TRY(call.operand(&wd, w, c->w, sizeof(float2) * (size_t)c->T * c->M, z_out, vb, b_out));
+  const bool apart = !overlap(z_out, vb, b_out, vb);
+  const bool zdir = apart && in_place(c, z_out), bdir = apart && in_place(c, b_out);
+  float2* b = bdir ? (float2*)b_out : (b_out ? c->b : nullptr);
+  CISOR_TRY(sense_adjoint(c, fd, wd, zdir ? (float2*)z_out : c->z, b, c->T));
+  if (!zdir) CISOR_TRY(call.out(z_out, c->z, vb));
+  if (!bdir) CISOR_TRY(call.out(b_out, c->b, vb));
   return call.leave();
 }
 
@@ -589,8 +630,10 @@ cisor_status cisor_data_term(cisor_ctx* c, const void* f, const void* y, double*
   CISOR_TRY(call.in(c->yobs, y, sizeof(float2) * (size_t)c->T * c->M));
   double D = 0.0;
   cisor_solve_info li{};
-  cisor_status st = data_core(c, o, &D, &li);
+  cisor_status st = data_core(c, o, &li);
   if (!solve_ok(st)) return st;
+  CISOR_CUDA(cudaStreamSynchronize(c->stream));
+  D = c->h_dsum[0];
   c->have_w = 1;
   if (D_out) *D_out = D;
   if (info) *info = li;
@@ -634,10 +677,14 @@ static cisor_status tv_prox_entry(cisor_ctx* c, const void* z, void* x, double g
   }
   Call call(c);
   CISOR_TRY(call.enter());
-  CISOR_TRY(call.in(c->fz, z, sizeof(float2) * c->N));
+  const size_t nb = sizeof(float2) * c->N;
+  const float2* zd;
+  CISOR_TRY(call.operand(&zd, z, c->fz, nb, x, nb));
+  const bool direct = in_place(c, x);
   auto prox = aniso ? tv_prox_aniso : tv_prox;
-  CISOR_TRY(prox(c, c->fz, c->work_n, gamma_tau, iters, lo, hi, lo_im, hi_im, c->complex_f, nullptr, 0.0, nullptr));
-  CISOR_TRY(call.out(x, c->work_n, sizeof(float2) * c->N));
+  CISOR_TRY(prox(c, zd, direct ? (float2*)x : c->work_n, gamma_tau, iters, lo, hi, lo_im, hi_im, c->complex_f, nullptr,
+                 0.0, nullptr));
+  if (!direct) CISOR_TRY(call.out(x, c->work_n, nb));
   return call.leave();
 }
 
@@ -743,8 +790,6 @@ cisor_status cisor_set_rx_mask(cisor_ctx* c, const void* mask) {
   return call.leave();
 }
 
-static bool two_stage_ok(const cisor_ctx* c) { return c->P == 128 || c->P == 256 || (c->dim == 2 && c->P == 512); }
-
 cisor_status cisor_set_cols_cta(cisor_ctx* c, int cols_nt) {
   if (!c || (cols_nt != 512 && cols_nt != 256 && cols_nt != COLS_TWO_STAGE && cols_nt != COLS_CLUSTER)) {
     set_error("cisor_set_cols_cta: NULL context or cols_nt not 512 / 256 / %d / %d", COLS_TWO_STAGE, COLS_CLUSTER);
@@ -846,9 +891,9 @@ cisor_status cisor_autotune(cisor_ctx* c, int reps, int* cols_nt_out) {
     for (int h = 0; h < nch && st == CISOR_OK; ++h) {
       c->cols_nt = variants[v];
       c->tx_chunk = chunks[h];
-      st = matvec_once(c, 0, c->T, c->s, c->tv);  // warm-up
+      st = matvec_once(c, 0, c->T, c->f, c->s, c->tv);  // warm-up
       CISOR_CUDA(cudaEventRecord(e0, c->stream));
-      for (int i = 0; i < reps && st == CISOR_OK; ++i) st = matvec_once(c, 0, c->T, c->s, c->tv);
+      for (int i = 0; i < reps && st == CISOR_OK; ++i) st = matvec_once(c, 0, c->T, c->f, c->s, c->tv);
       CISOR_CUDA(cudaEventRecord(e1, c->stream));
       CISOR_CUDA(cudaEventSynchronize(e1));
       float ms = 0.f;
@@ -900,13 +945,13 @@ cisor_status cisor_time_matvec(cisor_ctx* c, const void* f, int adjoint, int rep
   CISOR_TRY(call.enter());
   CISOR_TRY(call.in(c->f, f, sizeof(float2) * c->N));
   CISOR_CUDA(cudaMemcpyAsync(c->s, c->u_in, sizeof(float2) * (size_t)c->T * c->Nf, cudaMemcpyDeviceToDevice, c->stream));
-  CISOR_TRY(matvec_once(c, adjoint, c->T, c->s, c->tv));
+  CISOR_TRY(matvec_once(c, adjoint, c->T, c->f, c->s, c->tv));
   cudaEvent_t e0, e1;
   CISOR_CUDA(cudaEventCreate(&e0));
   CISOR_CUDA(cudaEventCreate(&e1));
   CISOR_CUDA(cudaEventRecord(e0, c->stream));
   cisor_status st = CISOR_OK;
-  for (int i = 0; i < reps && st == CISOR_OK; ++i) st = matvec_once(c, adjoint, c->T, c->s, c->tv);
+  for (int i = 0; i < reps && st == CISOR_OK; ++i) st = matvec_once(c, adjoint, c->T, c->f, c->s, c->tv);
   CISOR_CUDA(cudaEventRecord(e1, c->stream));
   CISOR_CUDA(cudaEventSynchronize(e1));
   float ms = 0.f;

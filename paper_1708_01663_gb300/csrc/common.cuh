@@ -86,6 +86,13 @@ enum { TX_OK = 0, TX_BREAKDOWN = 1, TX_MAXITER = 2 };
 
 }  // namespace cisor
 
+// A transmitter's solve status in mapped host memory: kernels store it when it
+// changes and the host reads it after waiting for the stream, with no copy.
+struct cisor_txstat {
+  double rel;  // true relative residual
+  int active, iters, flag, pad;
+};
+
 struct cisor_ctx {
   // geometry
   int dim, n, P, T, M, complex_f;
@@ -133,7 +140,8 @@ struct cisor_ctx {
   int nblk;        // dot partials per transmitter
   double* scal;    // [T, SC_STRIDE] double2
   int *active, *iters, *txflag;
-  int* h_active;    // pinned [T]
+  cisor_txstat *h_stat, *stat;  // mapped host [T] and its device alias
+  double sp_tol, sp_max_iter;   // the solve parameters in sparams
   double* dsum;     // device scalar accumulators [4]
   double* h_dsum;   // pinned [4]
   // TV workspace (d dual components x N floats per plane, up to 2 planes)
@@ -311,6 +319,7 @@ cisor_status adjoint_fields(cisor_ctx* c);  // c->gz = c->z + G^H c->vadj unless
 // [T][3 nblk][DOT_SLOTS].
 struct VecOp {
   int adjoint, epilogue;  // EPI_MATVEC or EPI_RESID
+  const float2* f;        // [N]
   const float2* x;        // input (and the x of A x)
   const float2* aux;      // b of EPI_RESID, dot operand
   float2* out;

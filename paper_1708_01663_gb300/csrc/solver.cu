@@ -37,7 +37,8 @@ enum { SCM_INIT = 0, SCM_ALPHA = 1, SCM_OMEGA = 2, SCM_RHO = 3, SCM_TRUE = 4 };
 __global__ void __launch_bounds__(32) bicg_scalar_kernel(int mode, int nblk, const float* __restrict__ part,
                                                          double* __restrict__ scal, int* __restrict__ active,
                                                          int* __restrict__ iters, int* __restrict__ txflag,
-                                                         const double* __restrict__ params) {
+                                                         const double* __restrict__ params,
+                                                         cisor_txstat* __restrict__ stat) {
   pdl_trigger();
   pdl_wait();
   const int t = blockIdx.x, lane = threadIdx.x;
@@ -58,6 +59,7 @@ __global__ void __launch_bounds__(32) bicg_scalar_kernel(int mode, int nblk, con
   const double2 d0 = make_double2(d[0], d[1]), d1 = make_double2(d[2], d[3]), d2 = make_double2(d[4], d[5]);
   double2* sc = reinterpret_cast<double2*>(scal) + (size_t)t * SC_STRIDE;
   int act = active[t];
+  const int was = act;
   if (mode == SCM_INIT) {
     const double bn2 = d0.x, rn2 = d2.x;
     const double rel = bn2 > 0.0 ? sqrt(rn2 / bn2) : 0.0;
@@ -131,6 +133,8 @@ __global__ void __launch_bounds__(32) bicg_scalar_kernel(int mode, int nblk, con
     }
   }
   active[t] = act;
+  if (mode == SCM_INIT || mode == SCM_TRUE || act != was)
+    stat[t] = cisor_txstat{sc[SC_REL].y, act, iters[t], txflag[t], 0};
 }
 
 // x += alpha p + omega s ; r = s - omega t ; partials <rhat, r> (slot 0), <r, r> (slot 2).
@@ -235,7 +239,8 @@ __global__ void __launch_bounds__(256) bicg_zero_start_kernel(int n, int nrows, 
 
 static cisor_status scalar_step(cisor_ctx* c, int mode, int ntx) {
   (void)launch_pdl(bicg_scalar_kernel, dim3(ntx), dim3(32), 0, c->stream, mode, c->nblk * c->ncomp,
-                   (const float*)c->part, c->scal, c->active, c->iters, c->txflag, (const double*)c->sparams);
+                   (const float*)c->part, c->scal, c->active, c->iters, c->txflag, (const double*)c->sparams,
+                   c->stat);
   CISOR_CUDA(cudaGetLastError());
   c->launches += 1;
   return CISOR_OK;
@@ -257,6 +262,7 @@ static ConvOp base_op(cisor_ctx* c, int adjoint, int ntx) {
 static cisor_status residual_pass(cisor_ctx* c, int adjoint, const float2* b, const float2* x, int ntx, bool gz) {
   if (c->ncomp == 3) {
     VecOp vo{};
+    vo.f = c->f;
     vo.adjoint = adjoint;
     vo.epilogue = EPI_RESID;
     vo.x = x;
@@ -306,6 +312,7 @@ static cisor_status update_step(cisor_ctx* c, float2* x, int ntx) {
 static cisor_status enqueue_iteration_vec(cisor_ctx* c, int adjoint, float2* x, int ntx) {
   CISOR_TRY(vec_pupdate(c, ntx));
   VecOp op{};
+  op.f = c->f;
   op.adjoint = adjoint;
   op.epilogue = EPI_MATVEC;
   op.x = c->p;
@@ -319,6 +326,7 @@ static cisor_status enqueue_iteration_vec(cisor_ctx* c, int adjoint, float2* x, 
   CISOR_TRY(scalar_step(c, SCM_ALPHA, ntx));
   CISOR_TRY(vec_axpy(c, ntx));
   VecOp op2{};
+  op2.f = c->f;
   op2.adjoint = adjoint;
   op2.epilogue = EPI_MATVEC;
   op2.x = c->s;
@@ -525,26 +533,29 @@ static cisor_status get_while_graph(cisor_ctx* c, int adjoint, float2* x, int nt
   return CISOR_OK;
 }
 
-static cisor_status read_active(cisor_ctx* c, int ntx, int* n_active) {
-  CISOR_CUDA(cudaMemcpyAsync(c->h_active, c->active, sizeof(int) * ntx, cudaMemcpyDeviceToHost, c->stream));
-  CISOR_CUDA(cudaStreamSynchronize(c->stream));
+// transmitters still active, once c's stream has been waited for
+static int count_active(const cisor_ctx* c, int ntx) {
   int s = 0;
-  for (int t = 0; t < ntx; ++t) s += c->h_active[t];
-  *n_active = s;
+  for (int t = 0; t < ntx; ++t) s += ((volatile const cisor_txstat*)c->h_stat)[t].active;
+  return s;
+}
+static cisor_status read_active(cisor_ctx* c, int ntx, int* n_active) {
+  CISOR_CUDA(cudaStreamSynchronize(c->stream));
+  *n_active = count_active(c, ntx);
   return CISOR_OK;
 }
 
-// Sets the solve parameters, zeroes p and v, forms r = b - A x0, rhat = r and
-// runs the INIT scalar step (all on c->stream).
+// Sets the solve parameters, forms r = b - A x0, rhat = r and runs the INIT scalar step (all on c->stream).  p and v
+// need no initial value: INIT sets beta = 0, with which the first iteration takes p = r.
 static cisor_status init_solve(cisor_ctx* c, int adjoint, const float2* b, float2* x, int x_zero, int ntx,
                                double tol, int max_iter) {
-  const size_t vb = sizeof(float2) * (size_t)ntx * c->Nf;
-  // pageable source: the copy is staged before cudaMemcpyAsync returns, so the stack array may go
-  const double hp[2] = {tol, (double)max_iter};
-  CISOR_CUDA(cudaMemcpyAsync(c->sparams, hp, sizeof(hp), cudaMemcpyHostToDevice, c->stream));
-  CISOR_CUDA(cudaMemsetAsync(c->p, 0, vb, c->stream));
-  CISOR_CUDA(cudaMemsetAsync(c->v, 0, vb, c->stream));
-  CISOR_CUDA(cudaMemsetAsync(c->active, 0, sizeof(int) * ntx, c->stream));
+  if (c->sp_tol != tol || c->sp_max_iter != (double)max_iter) {
+    // pageable source: the copy is staged before cudaMemcpyAsync returns, so the stack array may go
+    const double hp[2] = {tol, (double)max_iter};
+    CISOR_CUDA(cudaMemcpyAsync(c->sparams, hp, sizeof(hp), cudaMemcpyHostToDevice, c->stream));
+    c->sp_tol = tol;
+    c->sp_max_iter = max_iter;
+  }
   if (adjoint) c->gz_ready = 0;
   if (x_zero) {
     CISOR_CUDA(launch_pdl(bicg_zero_start_kernel, dim3(c->nblk * c->ncomp, ntx), dim3(256), 0, c->stream, c->n,
@@ -568,29 +579,25 @@ static cisor_status true_residual(cisor_ctx* c, int adjoint, const float2* b, fl
 // transmitter above tol (breakdown or iteration cap).
 static cisor_status collect_stats(cisor_ctx* c, int adjoint, int ntx, double tol, int* iters_max,
                                   double* iters_mean, double* resid_max, int* n_bad) {
-  std::vector<int> it(ntx), fl(ntx);
-  std::vector<double> sc((size_t)ntx * SC_STRIDE * 2);
-  CISOR_CUDA(cudaMemcpyAsync(it.data(), c->iters, sizeof(int) * ntx, cudaMemcpyDeviceToHost, c->stream));
-  CISOR_CUDA(cudaMemcpyAsync(fl.data(), c->txflag, sizeof(int) * ntx, cudaMemcpyDeviceToHost, c->stream));
-  CISOR_CUDA(cudaMemcpyAsync(sc.data(), c->scal, sizeof(double) * sc.size(), cudaMemcpyDeviceToHost, c->stream));
-  CISOR_CUDA(cudaStreamSynchronize(c->stream));
-  c->last_iters[adjoint ? 1 : 0] = it;
-  int imax = 0, bad = 0;
+  const volatile cisor_txstat* st = c->h_stat;  // the caller has waited for the stream
+  std::vector<int>& it = c->last_iters[adjoint ? 1 : 0];
+  it.resize(ntx);
+  int imax = 0, bad = 0, brk = 0;
   double isum = 0.0, rmax = 0.0;
   for (int t = 0; t < ntx; ++t) {
+    it[t] = st[t].iters;
     imax = it[t] > imax ? it[t] : imax;
     isum += it[t];
-    const double rel = sc[((size_t)t * SC_STRIDE + SC_REL) * 2 + 1];
+    const double rel = st[t].rel;
     rmax = (rel > rmax || !(rel == rel)) ? rel : rmax;
     if (!(rel <= tol)) ++bad;
+    brk |= st[t].flag == TX_BREAKDOWN;
   }
   if (iters_max) *iters_max = imax;
   if (iters_mean) *iters_mean = isum / (ntx > 0 ? ntx : 1);
   if (resid_max) *resid_max = rmax;
   if (n_bad) *n_bad = bad;
   if (bad) {
-    int brk = 0;
-    for (int t = 0; t < ntx; ++t) brk |= (fl[t] == TX_BREAKDOWN);
     set_error("%d of %d field solves above tol %.3g (max true residual %.3g)%s", bad, ntx, tol, rmax,
               brk ? ", Krylov breakdown" : "");
     return brk ? CISOR_ERR_BREAKDOWN : CISOR_ERR_NOT_CONVERGED;
@@ -642,13 +649,11 @@ cisor_status solve_multi(cisor_ctx* const* cs, int np, int adjoint, const float2
   for (int i = 0; i < np; ++i)
     CISOR_TRY(init_solve(cs[i], adjoint, b[i], xof(cs[i]), x_zero ? x_zero[i] : 0, cs[i]->T, tol, max_iter));
   auto count = [&](int* total) -> cisor_status {
-    for (int i = 0; i < np; ++i)
-      CISOR_CUDA(cudaMemcpyAsync(cs[i]->h_active, cs[i]->active, sizeof(int) * cs[i]->T, cudaMemcpyDeviceToHost,
-                                 cs[i]->stream));
     int s = 0;
     for (int i = 0; i < np; ++i) {
-      CISOR_CUDA(cudaStreamSynchronize(cs[i]->stream));
-      for (int t = 0; t < cs[i]->T; ++t) s += cs[i]->h_active[t];
+      int k = 0;
+      CISOR_TRY(read_active(cs[i], cs[i]->T, &k));
+      s += k;
     }
     *total = s;
     return CISOR_OK;

@@ -149,7 +149,7 @@ cisor_status vec_matvec(cisor_ctx* c, const VecOp& op) {
     co.src = op.x;
     co.epilogue = EPI_CONV_ADD;
     co.out = c->vbuf;
-    co.f = c->f;
+    co.f = op.f;
     co.ntx = 3 * op.ntx;
     co.tx_div = 3;
     co.active = op.active;
@@ -191,7 +191,7 @@ cisor_status vec_matvec(cisor_ctx* c, const VecOp& op) {
     co.dot_b[s] = op.dot_b[s];
   }
   co.part = c->part;
-  co.f = c->f;
+  co.f = op.f;
   co.ntx = 3 * op.ntx;
   co.tx_div = 3;
   co.active = op.active;
