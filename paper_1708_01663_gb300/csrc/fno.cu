@@ -114,7 +114,8 @@ __device__ __forceinline__ uint32_t bf_bits(__nv_bfloat16 h) { return (uint32_t)
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uint32_t& lo) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);  // one packed conversion, x0 in the low half
   const float2 hf = __bfloat1622float2(h);
-  const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - hf.x, x1 - hf.y);
+  const float2 d = pair_sub(make_float2(x0, x1), hf);
+  const __nv_bfloat162 l = __floats2bfloat162_rn(d.x, d.y);
   hi = *reinterpret_cast<const uint32_t*>(&h);
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
@@ -559,21 +560,22 @@ __global__ void __launch_bounds__(NTH, 2) fno_row_tc(const float* __restrict__ v
     // epilogue: pre = D + b (to global when training), v_{l+1} = act(pre) to global, staged as the next A
     float v[FC];
     tmem_ld32(tl + 32 * r, v);
-#pragma unroll
-    for (int j = 0; j < FC / 4; ++j) {
-      const float4 bj = reinterpret_cast<const float4*>(bias)[j];
-      v[4 * j] += bj.x;
-      v[4 * j + 1] += bj.y;
-      v[4 * j + 2] += bj.z;
-      v[4 * j + 3] += bj.w;
-    }
     {
       const long long g0 = gbase + (long long)r * FN + ix;
 #pragma unroll
-      for (int c = 0; c < FC; ++c) {
-        if (pre_out) pre_out[g0 + (long long)c * FNN] = v[c];
-        if (act) v[c] = gelu_f(v[c]);
-        if (vout) vout[g0 + (long long)c * FNN] = v[c];
+      for (int c = 0; c < FC; c += 2) {
+        float2 x = pair_add(make_float2(v[c], v[c + 1]), *reinterpret_cast<const float2*>(bias + c));
+        if (pre_out) {
+          pre_out[g0 + (long long)c * FNN] = x.x;
+          pre_out[g0 + (long long)(c + 1) * FNN] = x.y;
+        }
+        if (act) x = gelu_f(x);
+        if (vout) {
+          vout[g0 + (long long)c * FNN] = x.x;
+          vout[g0 + (long long)(c + 1) * FNN] = x.y;
+        }
+        v[c] = x.x;
+        v[c + 1] = x.y;
       }
     }
     if (!PROJ) {
@@ -632,7 +634,7 @@ __global__ void __launch_bounds__(NTH, 2) fno_row_tc(const float* __restrict__ v
           dst[(ky * FC + (rr & 31)) * RB + (rr >> 5)] = make_float2(d[2 * k], d[2 * k + 1]);
         }
     } else {  // out = P2 GELU(z + c1) + c2 for this thread's pixel; warm start x0 = u_in (1 + out)
-      float o0 = c20, o1 = c21;
+      float2 o0 = make_float2(c20, 0.f), o1 = make_float2(c21, 0.f);  // even and odd hidden units
       const float4 *c14 = reinterpret_cast<const float4*>(c1), *p204 = reinterpret_cast<const float4*>(p2),
                    *p214 = reinterpret_cast<const float4*>(p2 + FH);
 #pragma unroll 1
@@ -642,14 +644,14 @@ __global__ void __launch_bounds__(NTH, 2) fno_row_tc(const float* __restrict__ v
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const float4 cc = c14[8 * j + k], q0 = p204[8 * j + k], q1 = p214[8 * j + k];
-          const float h0 = gelu_f(d[4 * k] + cc.x), h1 = gelu_f(d[4 * k + 1] + cc.y);
-          const float h2 = gelu_f(d[4 * k + 2] + cc.z), h3 = gelu_f(d[4 * k + 3] + cc.w);
-          o0 += q0.x * h0 + q0.y * h1 + q0.z * h2 + q0.w * h3;
-          o1 += q1.x * h0 + q1.y * h1 + q1.z * h2 + q1.w * h3;
+          const float2 h0 = gelu_f(pair_add(make_float2(d[4 * k], d[4 * k + 1]), make_float2(cc.x, cc.y)));
+          const float2 h1 = gelu_f(pair_add(make_float2(d[4 * k + 2], d[4 * k + 3]), make_float2(cc.z, cc.w)));
+          o0 = pair_fma(make_float2(q0.z, q0.w), h1, pair_fma(make_float2(q0.x, q0.y), h0, o0));
+          o1 = pair_fma(make_float2(q1.z, q1.w), h1, pair_fma(make_float2(q1.x, q1.y), h0, o1));
         }
       }
       const long long pix = (long long)b * FNN + pix0 + (long long)r * FN + ix;
-      const float2 e = make_float2(o0, o1);
+      const float2 e = make_float2(o0.x + o0.y, o1.x + o1.y);
       if (out) out[pix] = e;
       if (x0) {
         const float2 u = u_in[pix];
@@ -949,10 +951,9 @@ __global__ void __launch_bounds__(NTH, 2) fno_row_bwd(const float* __restrict__ 
     if (act)
       planar_pass(gs, gbase, [&](float4& x, long long gi) {
         const float4 p = *reinterpret_cast<const float4*>(pre + gi);
-        x.x *= gelu_grad_f(p.x);
-        x.y *= gelu_grad_f(p.y);
-        x.z *= gelu_grad_f(p.z);
-        x.w *= gelu_grad_f(p.w);
+        const float2 a = pair_mul(make_float2(x.x, x.y), gelu_grad_f(make_float2(p.x, p.y)));
+        const float2 b = pair_mul(make_float2(x.z, x.w), gelu_grad_f(make_float2(p.z, p.w)));
+        x = make_float4(a.x, a.y, b.x, b.y);
       });
     __syncthreads();
     // dvp_out = W^T dpre: GEMM M = NP, N = FC (i), K = FC (o)
@@ -1052,14 +1053,17 @@ __global__ void __launch_bounds__(NTH, 1) fno_proj_bwd(const float* __restrict__
           mma2(d, av[h][0], b0);
           mma2(d, av[h][1], b1);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int p = 16 * mt + g + (e >> 1) * 8, hl = 8 * nt + 2 * t + (e & 1), hid = 32 * q + hl;
-            const float z = d[e] + c1[hid];
-            const float dh = p2[hid] * ds[p] + p2[FH + hid] * ds[NPP + p];
-            float gv, gd;
-            gelu_and_grad(z, gv, gd);
-            hs[hl * NPP + p] = gv;
-            zs[hl * NPP + p] = dh * gd;
+          for (int e = 0; e < 2; ++e) {  // rows g and g + 8 of the tile, two consecutive hidden units each
+            const int p = 16 * mt + g + e * 8, hl = 8 * nt + 2 * t, hid = 32 * q + hl;
+            const float2 z = pair_add(make_float2(d[2 * e], d[2 * e + 1]), *reinterpret_cast<const float2*>(c1 + hid));
+            const float2 dh = pair_fma(*reinterpret_cast<const float2*>(p2 + FH + hid), pair_of(ds[NPP + p]),
+                                       pair_mul(*reinterpret_cast<const float2*>(p2 + hid), pair_of(ds[p])));
+            float2 gv;
+            const float2 dz = pair_mul(dh, gelu_and_grad(z, gv));
+            hs[hl * NPP + p] = gv.x;
+            hs[(hl + 1) * NPP + p] = gv.y;
+            zs[hl * NPP + p] = dz.x;
+            zs[(hl + 1) * NPP + p] = dz.y;
           }
         }
       }

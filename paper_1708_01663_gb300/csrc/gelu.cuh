@@ -30,39 +30,76 @@ __host__ __device__ __forceinline__ float gelu_exp(float x) {
 #endif
 }
 
+// Two values at once: on the device the pair's sums, products and multiply-adds are single packed instructions of
+// the sm_100 family (same rounding, half the issue slots; the FNO's row kernels are bound by issue in these
+// functions).  The host build computes the halves one by one.
+__host__ __device__ __forceinline__ float2 pair_fma(float2 a, float2 b, float2 c) {
+#ifdef __CUDA_ARCH__
+  return __ffma2_rn(a, b, c);
+#else
+  return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
+#endif
+}
+__host__ __device__ __forceinline__ float2 pair_mul(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+  return __fmul2_rn(a, b);
+#else
+  return make_float2(a.x * b.x, a.y * b.y);
+#endif
+}
+__host__ __device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+  return __fadd2_rn(a, b);
+#else
+  return make_float2(a.x + b.x, a.y + b.y);
+#endif
+}
+__host__ __device__ __forceinline__ float2 pair_of(float a) { return make_float2(a, a); }
+__host__ __device__ __forceinline__ float2 pair_sub(float2 a, float2 b) { return pair_fma(b, pair_of(-1.f), a); }
+
 // erf(z) for z >= 0
-__host__ __device__ __forceinline__ float erf_pos(float z) {
-  z = fminf(z, 4.f);
-  float p = fmaf(4.30638e-5f, z, 2.765672e-4f);
-  p = fmaf(p, z, 1.520143e-4f);
-  p = fmaf(p, z, 9.2705272e-3f);
-  p = fmaf(p, z, 4.22820123e-2f);
-  p = fmaf(p, z, 7.05230784e-2f);
-  p = fmaf(p, z, 1.f);
-  p *= p;
-  p *= p;
-  p *= p;
-  p *= p;
-  return 1.f - gelu_rcp(p);
+__host__ __device__ __forceinline__ float2 erf_pos(float2 z) {
+  z = make_float2(fminf(z.x, 4.f), fminf(z.y, 4.f));
+  float2 p = pair_fma(pair_of(4.30638e-5f), z, pair_of(2.765672e-4f));
+  p = pair_fma(p, z, pair_of(1.520143e-4f));
+  p = pair_fma(p, z, pair_of(9.2705272e-3f));
+  p = pair_fma(p, z, pair_of(4.22820123e-2f));
+  p = pair_fma(p, z, pair_of(7.05230784e-2f));
+  p = pair_fma(p, z, pair_of(1.f));
+  p = pair_mul(p, p);
+  p = pair_mul(p, p);
+  p = pair_mul(p, p);
+  p = pair_mul(p, p);
+  return pair_sub(pair_of(1.f), make_float2(gelu_rcp(p.x), gelu_rcp(p.y)));
 }
 
-__host__ __device__ __forceinline__ float gelu_f(float x) {
-  const float a = fabsf(x);
-  return 0.5f * fmaf(a, erf_pos(a * 0.70710678118654752f), x);
+__host__ __device__ __forceinline__ float2 gelu_f(float2 x) {
+  const float2 a = make_float2(fabsf(x.x), fabsf(x.y));
+  return pair_mul(pair_of(0.5f), pair_fma(a, erf_pos(pair_mul(a, pair_of(0.70710678118654752f))), x));
 }
 
-__host__ __device__ __forceinline__ float gelu_grad_f(float x) {
-  const float e = erf_pos(fabsf(x) * 0.70710678118654752f);
-  const float phi = 0.5f * (1.f + copysignf(e, x));
-  return fmaf(x * 0.39894228040143268f, gelu_exp(-0.5f * x * x), phi);
+// both at once (one erf): g = gelu(x), the result gelu'(x)
+__host__ __device__ __forceinline__ float2 gelu_and_grad(float2 x, float2& g) {
+  const float2 a = make_float2(fabsf(x.x), fabsf(x.y));
+  const float2 e = erf_pos(pair_mul(a, pair_of(0.70710678118654752f)));
+  g = pair_mul(pair_of(0.5f), pair_fma(a, e, x));
+  const float2 h = pair_mul(pair_mul(x, pair_of(-0.5f)), x);
+  const float2 phi = pair_fma(make_float2(copysignf(e.x, x.x), copysignf(e.y, x.y)), pair_of(0.5f), pair_of(0.5f));
+  return pair_fma(pair_mul(x, pair_of(0.39894228040143268f)), make_float2(gelu_exp(h.x), gelu_exp(h.y)), phi);
+}
+__host__ __device__ __forceinline__ float2 gelu_grad_f(float2 x) {
+  float2 g;
+  return gelu_and_grad(x, g);
 }
 
-// both at once (one erf): g = gelu(x), gp = gelu'(x)
+// one value
+__host__ __device__ __forceinline__ float erf_pos(float z) { return erf_pos(make_float2(z, z)).x; }
+__host__ __device__ __forceinline__ float gelu_f(float x) { return gelu_f(make_float2(x, x)).x; }
+__host__ __device__ __forceinline__ float gelu_grad_f(float x) { return gelu_grad_f(make_float2(x, x)).x; }
 __host__ __device__ __forceinline__ void gelu_and_grad(float x, float& g, float& gp) {
-  const float a = fabsf(x);
-  const float e = erf_pos(a * 0.70710678118654752f);
-  g = 0.5f * fmaf(a, e, x);
-  gp = fmaf(x * 0.39894228040143268f, gelu_exp(-0.5f * x * x), 0.5f * (1.f + copysignf(e, x)));
+  float2 g2;
+  gp = gelu_and_grad(make_float2(x, x), g2).x;
+  g = g2.x;
 }
 
 }  // namespace cisor
