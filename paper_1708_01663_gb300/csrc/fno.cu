@@ -337,6 +337,13 @@ __device__ __forceinline__ void planar_pass(float* sm, long long gbase, Op op) {
   }
 }
 
+// Every kernel of a forward or backward pass is launched with programmatic stream serialization (pdl_wait): it
+// takes its tensor memory, copies the DFT tables and weights to shared memory and only then waits for the kernel
+// before it.  Tables and weights do not change within a pass, and the copies of a pass's inputs separate it from the
+// kernels that write weights.  A kernel triggers its dependents after its own tensor-memory allocation, so all CTAs of
+// a kernel hold theirs before any CTA of the next can ask for columns: the next kernel may wait for columns, never
+// the other way round.  Inference of 32 samples 421 -> 380 us, loss and gradients 1464 -> 1388 us.
+
 // ------------------------------------------------------------------ forward kernels
 // v0 = W0 a + b0 (lifting), v0 to global, and its row DFT (the first column kernel's input).
 constexpr int SM_LIFT = (FC * NPP + FIN * NPP) * 4 + ((RB + 2) * FN + NP + BLK) * 8 + T_ROW * 2;
@@ -356,10 +363,12 @@ __global__ void __launch_bounds__(NTH, 2) fno_lift_fwd(const float2* __restrict_
   __shared__ __nv_bfloat16 w0[FC * FIN];
   __shared__ float b0[FC];
   const int b = blockIdx.y, iyb = blockIdx.x, iy0 = iyb * RB;
-  load_inputs(u_in, f, fps, b, iy0, us, fs);
+  pdl_trigger();
   cta_copy(tb, tabs, T_ROW * 2);
   for (int i = threadIdx.x; i < FC * FIN; i += NTH) w0[i] = wbf[F_W0 + i];
   if (threadIdx.x < FC) b0[threadIdx.x] = pm[F_B0 + threadIdx.x];
+  pdl_wait();
+  load_inputs(u_in, f, fps, b, iy0, us, fs);
   cp_wait_all();
   __syncthreads();
   features(us, fs, iy0, as);
@@ -465,6 +474,7 @@ __global__ void __launch_bounds__(NTH, 2) fno_row_tc(const float* __restrict__ v
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_trigger();
   const uint32_t tmem = tslot;
   const uint32_t s0 = smem_addr(sm);
   const uint32_t tl = tmem + ((uint32_t)(32 * q4) << 16);  // this warp's TMEM lane quarter
@@ -514,6 +524,7 @@ __global__ void __launch_bounds__(NTH, 2) fno_row_tc(const float* __restrict__ v
   };
   const uint32_t id_i = tc_idesc_bf16(128, 64), id_w = tc_idesc_bf16(128, 32), id_f = tc_idesc_bf16(64, 32),
                  id_p = tc_idesc_bf16(128, 128);
+  pdl_wait();
   fetch(blockIdx.x);
   for (int it = blockIdx.x; it < items; it += gridDim.x) {
     const int b = it / NIB, iyb = it % NIB, iy0 = iyb * RB;
@@ -717,6 +728,11 @@ __global__ void __launch_bounds__(NTH, 1) fno_colf_tc(const float2* __restrict__
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ky0 = blockIdx.x * KY_G, b = blockIdx.y;
   cta_copy(sm + 2 * KCF_PA, tabs + T_TCOLF, 2 * KC_PB);
+  if (tid == 0) mbar_init(&mbar);
+  if (warp == 0) tmem_alloc(&tslot, 64);
+  __syncthreads();
+  pdl_trigger();
+  pdl_wait();
   // T[n = 32 kyl + c][k = 2 iy + p]: one 16-byte load per (n, row pair) = k 4 iyb .. 4 iyb + 3.  A warp
   // covers 8 n x 4 row pairs: 128-byte global pieces, 8-byte stores on all 32 banks.
   const float2* tb = Tin + (long long)b * NIB * BLK + ky0 * FC * RB;
@@ -732,8 +748,6 @@ __global__ void __launch_bounds__(NTH, 1) fno_colf_tc(const float2* __restrict__
     *reinterpret_cast<uint2*>(sm + o) = h;
     *reinterpret_cast<uint2*>(sm + KCF_PA + o) = l;
   }
-  if (tid == 0) mbar_init(&mbar);
-  if (warp == 0) tmem_alloc(&tslot, 64);
   cp_wait_all();
   fence_async_smem();
   tc_fence_before();
@@ -784,6 +798,11 @@ __global__ void __launch_bounds__(NTH, 2) fno_coli_tc(const float2* __restrict__
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ky0 = blockIdx.x * KY_G, b = blockIdx.y;
   cta_copy(sm + 2 * KCI_PA, tabs + T_TCOLI, 2 * KC_PB);
+  if (tid == 0) mbar_init(&mbar);
+  if (warp == 0) tmem_alloc(&tslot, 256);
+  __syncthreads();
+  pdl_trigger();
+  pdl_wait();
   // Y[n = 32 kyl + o][k = 2 kx + p]: a warp covers 8 n x 4 kx (64-byte global pieces, 4-byte stores on
   // all 32 banks)
 #pragma unroll 8
@@ -797,8 +816,6 @@ __global__ void __launch_bounds__(NTH, 2) fno_coli_tc(const float2* __restrict__
     *reinterpret_cast<uint32_t*>(sm + o) = h;
     *reinterpret_cast<uint32_t*>(sm + KCI_PA + o) = l;
   }
-  if (tid == 0) mbar_init(&mbar);
-  if (warp == 0) tmem_alloc(&tslot, 256);
   cp_wait_all();
   fence_async_smem();
   tc_fence_before();
@@ -843,7 +860,9 @@ __global__ void __launch_bounds__(NTH) fno_mix(const float2* __restrict__ X, con
   __shared__ float2 rs[FC * MIXP], xs[32 * MIXP];
   const int m = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const __nv_bfloat162* R = reinterpret_cast<const __nv_bfloat162*>(wbf + roff) + (long long)m * FC * FC;
+  pdl_trigger();
   for (int e = threadIdx.x; e < FC * FC; e += NTH) rs[(e / FC) * MIXP + e % FC] = __bfloat1622float2(R[e]);
+  pdl_wait();
   const float sc = ky_scale(m % FM);
   for (int b0 = 0; b0 < B; b0 += 32) {
     __syncthreads();
@@ -876,7 +895,9 @@ __global__ void __launch_bounds__(NTH) fno_mix_bwd(const float2* __restrict__ X,
   __shared__ float2 rs[FC * MIXP], xs[32 * MIXP], gs[32 * MIXP];
   const int m = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const __nv_bfloat162* R = reinterpret_cast<const __nv_bfloat162*>(wbf + roff) + (long long)m * FC * FC;
+  pdl_trigger();
   for (int e = threadIdx.x; e < FC * FC; e += NTH) rs[(e / FC) * MIXP + e % FC] = __bfloat1622float2(R[e]);
+  pdl_wait();
   float2 gr[4] = {};
   for (int b0 = 0; b0 < B; b0 += 32) {
     __syncthreads();
@@ -930,8 +951,10 @@ __global__ void __launch_bounds__(NTH, 2) fno_row_bwd(const float* __restrict__ 
   __nv_bfloat16* tb = reinterpret_cast<__nv_bfloat16*>(zs + BLK);  // [T_ROW]
   __nv_bfloat16* wt = tb + T_ROW;                          // [FC][WP]: W^T (i, o)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  pdl_trigger();
   cta_copy(tb, tabs, T_ROW * 2);
   load_w(wbf + woff, nullptr, wt);
+  pdl_wait();
   float dw[4] = {0.f, 0.f, 0.f, 0.f};
   float db = 0.f;
   const int items = B * NIB;
@@ -1010,6 +1033,8 @@ __global__ void __launch_bounds__(NTH, 1) fno_proj_bwd(const float* __restrict__
   }
   for (int i = threadIdx.x; i < FH; i += NTH) c1[i] = pm[F_C1 + i];
   for (int i = threadIdx.x; i < 2 * FH; i += NTH) p2[i] = __bfloat162float(wbf[F_P2 + i]);
+  pdl_trigger();
+  pdl_wait();
   const uint32_t* p132 = reinterpret_cast<const uint32_t*>(p1);
   const uint32_t* p1t32 = reinterpret_cast<const uint32_t*>(p1t);
   float ap1[4][4];
@@ -1162,7 +1187,9 @@ __global__ void __launch_bounds__(NTH, 2) fno_lift_bwd(const float* __restrict__
   __nv_bfloat16* tb = reinterpret_cast<__nv_bfloat16*>(zs + BLK);  // [T_ROW]
   __shared__ float red[NTH / 32][4][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  pdl_trigger();
   cta_copy(tb, tabs, T_ROW * 2);
+  pdl_wait();
   float dw[4] = {0.f, 0.f, 0.f, 0.f};
   float db = 0.f;
   const int items = B * NIB;
@@ -1214,6 +1241,8 @@ __global__ void __launch_bounds__(32 * RED_W) fno_reduce(const float* __restrict
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;
   float s = 0.f;
+  pdl_trigger();
+  pdl_wait();
   if (i < count) {
 #pragma unroll 4
     for (int p = warp; p < nparts; p += RED_W) s += part[(long long)p * count + i];
@@ -1234,6 +1263,8 @@ __global__ void __launch_bounds__(256) fno_loss(const float2* __restrict__ out, 
   __shared__ float red[2][8];
   const long long b = blockIdx.x;
   float nd = 0.f, nt = 0.f;
+  pdl_trigger();
+  pdl_wait();
   for (int p = threadIdx.x; p < FNN; p += 256) {
     const float2 o = out[b * FNN + p], tv = t[b * FNN + p];
     const float dx = o.x - tv.x, dy = o.y - tv.y;
@@ -1435,26 +1466,22 @@ cisor_status fno_forward_core(cisor_fno* F, int fps, int B, int train, const flo
   cudaStream_t s = F->stream;
   const dim3 grow(NIB, B), gcol(FM / KY_G, B);
   const int gper = (int)((long long)B * NIB < F->grid_bwd ? (long long)B * NIB : F->grid_bwd);
-  fno_lift_fwd<<<grow, NTH, SM_LIFT, s>>>(F->fbuf, fps, xin, F->wbf, F->pm, F->tabs, F->v[0], F->T1);
-  CISOR_CUDA(cudaGetLastError());
+  CISOR_CUDA(launch_pdl(fno_lift_fwd, grow, dim3(NTH), SM_LIFT, s, F->fbuf, fps, xin, F->wbf, F->pm, F->tabs, F->v[0],
+                        F->T1));
   for (int l = 0; l < FL; ++l) {
     float2* X = train ? F->Xst[l] : F->Xsc;
-    fno_colf_tc<0><<<gcol, NTH, SM_COLF, s>>>(F->T1, F->tabs, B, X, F->dflag);
-    CISOR_CUDA(cudaGetLastError());
-    fno_mix<<<FMODES, NTH, 0, s>>>(X, F->wbf, f_R(l), B, F->Ysc);
-    CISOR_CUDA(cudaGetLastError());
-    fno_coli_tc<<<gcol, NTH, SM_COLI, s>>>(F->Ysc, F->tabs, B, F->Zb, F->dflag);
-    CISOR_CUDA(cudaGetLastError());
+    CISOR_CUDA(launch_pdl(fno_colf_tc<0>, gcol, dim3(NTH), SM_COLF, s, F->T1, F->tabs, B, X, F->dflag));
+    CISOR_CUDA(launch_pdl(fno_mix, dim3(FMODES), dim3(NTH), 0, s, X, F->wbf, f_R(l), B, F->Ysc));
+    CISOR_CUDA(launch_pdl(fno_coli_tc, gcol, dim3(NTH), SM_COLI, s, F->Ysc, F->tabs, B, F->Zb, F->dflag));
     const int last = l == FL - 1;
     float* pre = train ? F->pre[l] : nullptr;
     if (!last) {
-      fno_row_tc<0><<<gper, NTH, SM_ROW_TC, s>>>(F->v[l], F->Zb, F->wbf, F->pm, f_W(l), f_B(l), F->tabs, 1, B, pre,
-                                                 F->v[l + 1], F->T1, nullptr, nullptr, nullptr, F->dflag);
+      CISOR_CUDA(launch_pdl(fno_row_tc<0>, dim3(gper), dim3(NTH), SM_ROW_TC, s, F->v[l], F->Zb, F->wbf, F->pm, f_W(l),
+                            f_B(l), F->tabs, 1, B, pre, F->v[l + 1], F->T1, nullptr, nullptr, nullptr, F->dflag));
     } else {
-      fno_row_tc<1><<<gper, NTH, SM_ROW_TC, s>>>(F->v[l], F->Zb, F->wbf, F->pm, f_W(l), f_B(l), F->tabs, 0, B, pre,
-                                                 train ? F->v[FL] : nullptr, nullptr, F->out, xin, x0, F->dflag);
+      CISOR_CUDA(launch_pdl(fno_row_tc<1>, dim3(gper), dim3(NTH), SM_ROW_TC, s, F->v[l], F->Zb, F->wbf, F->pm, f_W(l),
+                            f_B(l), F->tabs, 0, B, pre, train ? F->v[FL] : nullptr, nullptr, F->out, xin, x0, F->dflag));
     }
-    CISOR_CUDA(cudaGetLastError());
   }
   return CISOR_OK;
 }
@@ -1465,34 +1492,30 @@ cisor_status fno_backward_core(cisor_fno* F, int fps, int B) {
   const int G = F->grid_bwd;
   const int Gi = (int)((long long)B * NIB < G ? (long long)B * NIB : G);
   const dim3 gcol(FM / KY_G, B);
-  fno_loss<<<B, 256, 0, s>>>(F->out, F->tbuf, B, F->dout, F->loss);
-  CISOR_CUDA(cudaGetLastError());
-  fno_proj_bwd<<<Gi, NTH, SM_PBWD, s>>>(F->v[FL], F->dout, F->wbf, F->pm, B, F->dvA, F->part);
-  CISOR_CUDA(cudaGetLastError());
-  fno_reduce<<<grid_of(PART_P, 32), 32 * RED_W, 0, s>>>(F->part, Gi, PART_P, F->grad + F_P1);
-  CISOR_CUDA(cudaGetLastError());
+  CISOR_CUDA(launch_pdl(fno_loss, dim3(B), dim3(256), 0, s, F->out, F->tbuf, B, F->dout, F->loss));
+  CISOR_CUDA(launch_pdl(fno_proj_bwd, dim3(Gi), dim3(NTH), SM_PBWD, s, F->v[FL], F->dout, F->wbf, F->pm, B, F->dvA,
+                        F->part));
+  CISOR_CUDA(launch_pdl(fno_reduce, dim3(grid_of(PART_P, 32)), dim3(32 * RED_W), 0, s, F->part, Gi, PART_P,
+                        F->grad + F_P1));
   float* dv = F->dvA;
   float* dvn = F->dvB;
   for (int l = FL - 1; l >= 0; --l) {
-    fno_row_bwd<<<Gi, NTH, SM_RBWD, s>>>(dv, l == FL - 1 ? nullptr : F->Zb, F->pre[l], F->v[l], F->wbf, f_W(l),
-                                         F->tabs, B, l < FL - 1, dvn, F->T1, F->part);
-    CISOR_CUDA(cudaGetLastError());
-    fno_reduce<<<grid_of(PART_W, 32), 32 * RED_W, 0, s>>>(F->part, Gi, PART_W, F->grad + f_W(l));
-    CISOR_CUDA(cudaGetLastError());
-    fno_colf_tc<1><<<gcol, NTH, SM_COLF, s>>>(F->T1, F->tabs, B, F->dYst, F->dflag);
-    CISOR_CUDA(cudaGetLastError());
-    fno_mix_bwd<<<FMODES, NTH, 0, s>>>(F->Xst[l], F->dYst, F->wbf, f_R(l), B, F->Xsc, F->grad + f_R(l));
-    CISOR_CUDA(cudaGetLastError());
-    fno_coli_tc<<<gcol, NTH, SM_COLI, s>>>(F->Xsc, F->tabs, B, F->Zb, F->dflag);
-    CISOR_CUDA(cudaGetLastError());
+    CISOR_CUDA(launch_pdl(fno_row_bwd, dim3(Gi), dim3(NTH), SM_RBWD, s, dv, l == FL - 1 ? nullptr : F->Zb, F->pre[l],
+                          F->v[l], F->wbf, f_W(l), F->tabs, B, l < FL - 1, dvn, F->T1, F->part));
+    CISOR_CUDA(launch_pdl(fno_reduce, dim3(grid_of(PART_W, 32)), dim3(32 * RED_W), 0, s, F->part, Gi, PART_W,
+                          F->grad + f_W(l)));
+    CISOR_CUDA(launch_pdl(fno_colf_tc<1>, gcol, dim3(NTH), SM_COLF, s, F->T1, F->tabs, B, F->dYst, F->dflag));
+    CISOR_CUDA(launch_pdl(fno_mix_bwd, dim3(FMODES), dim3(NTH), 0, s, F->Xst[l], F->dYst, F->wbf, f_R(l), B, F->Xsc,
+                          F->grad + f_R(l)));
+    CISOR_CUDA(launch_pdl(fno_coli_tc, gcol, dim3(NTH), SM_COLI, s, F->Xsc, F->tabs, B, F->Zb, F->dflag));
     float* tmp = dv;
     dv = dvn;
     dvn = tmp;
   }
-  fno_lift_bwd<<<Gi, NTH, SM_LBWD, s>>>(dv, F->Zb, F->fbuf, fps, F->ubuf, F->tabs, B, F->part);
-  CISOR_CUDA(cudaGetLastError());
-  fno_reduce<<<grid_of(PART_0, 32), 32 * RED_W, 0, s>>>(F->part, Gi, PART_0, F->grad + F_W0);
-  CISOR_CUDA(cudaGetLastError());
+  CISOR_CUDA(launch_pdl(fno_lift_bwd, dim3(Gi), dim3(NTH), SM_LBWD, s, dv, F->Zb, F->fbuf, fps, F->ubuf, F->tabs, B,
+                        F->part));
+  CISOR_CUDA(launch_pdl(fno_reduce, dim3(grid_of(PART_0, 32)), dim3(32 * RED_W), 0, s, F->part, Gi, PART_0,
+                        F->grad + F_W0));
   return CISOR_OK;
 }
 
