@@ -937,76 +937,235 @@ __global__ void __launch_bounds__(NTH) fno_mix_bwd(const float2* __restrict__ X,
 //   dpre = dv * GELU'(pre_l)      (or dv on the last layer)
 //   dvp_out = W_l^T dpre, dT = RowF(dpre),
 //   per-CTA partials of grad W_l = sum_p dpre v_l^T and grad b_l = sum_p dpre.
-constexpr int SM_RBWD = (2 * FC * NPP) * 4 + BLK * 8 + T_ROW * 2 + FC * WP * 2;
+// Warp w owns 16 pixels of each of the two image rows and all 32 channels: it forms RowI(dU) as tiles [16 channels]
+// [8 pixels], adds dvp and applies GELU' (both read from global memory in the tile's layout), and its registers then
+// hold dpre as the A fragments of grad W (K = its 16 pixels; v_l is read from global memory as B fragments, its 32 x
+// 32 accumulators stay in registers for the whole kernel) and, transposed by movmatrix, as the B fragments of W^T dpre.
+// Only dpre for RowF, whose sum runs over all pixels of a row, and dU go through shared memory, split once into BF16
+// hi / lo planes.  The version before staged all operands in FP32 in shared memory and split every fragment anew for
+// each product: 48.7 M instructions, 7 M bank conflicts and 103 us for 32 samples, now 25.2 M, 1 M and 78 us.  It now
+// waits for memory (issue 26 %): its four activation-sized streams take 39 us of HBM time, and 128 registers leave 16
+// warps an SM (asking for all of a row's operands before its first product spilled and gained nothing: 80 us).
+constexpr int RBZ = RIP * 2, RBP = RFP * 2;  // bytes of a row of the dU planes [64 rr][32 kyc] and of dpre [64 rr][128 ix]
+constexpr int RB_Z = T_ROW * 2, RB_P = RB_Z + 2 * 2 * FC * RBZ, RB_W = RB_P + 2 * 2 * FC * RBP, RB_T = RB_W + FC * WP * 2,
+              SM_RBWD = RB_T + BLK * 8;
+static_assert(SM_RBWD - RB_Z >= 8 * PART_W * 4, "the end of the kernel sums the warps' partials there");
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ uint32_t transpose8(uint32_t x) {
+  uint32_t y;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+  return y;
+}
 __global__ void __launch_bounds__(NTH, 2) fno_row_bwd(const float* __restrict__ dvp, const float2* __restrict__ dU,
                                                       const float* __restrict__ pre, const float* __restrict__ v,
                                                       const __nv_bfloat16* __restrict__ wbf, long long woff,
                                                       const __nv_bfloat16* __restrict__ tabs, int B, int act,
                                                       float* __restrict__ dvp_out, float2* __restrict__ dT,
                                                       float* __restrict__ part) {
-  extern __shared__ __align__(16) float smem[];
-  float* gs = smem;                                        // [FC][NPP] dv, then dpre
-  float* vs = gs + FC * NPP;                               // [FC][NPP] v_l
-  float2* zs = reinterpret_cast<float2*>(vs + FC * NPP);   // [BLK] dU block, then the dT block
-  __nv_bfloat16* tb = reinterpret_cast<__nv_bfloat16*>(zs + BLK);  // [T_ROW]
-  __nv_bfloat16* wt = tb + T_ROW;                          // [FC][WP]: W^T (i, o)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  extern __shared__ __align__(16) unsigned char sm[];
+  __nv_bfloat16* tb = reinterpret_cast<__nv_bfloat16*>(sm);            // [T_ROW] tables
+  __nv_bfloat16* wt = reinterpret_cast<__nv_bfloat16*>(sm + RB_W);     // [FC][WP]: W^T (i, o)
+  float2* stage = reinterpret_cast<float2*>(sm + RB_T);                // [BLK] the dT block
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+  const int j8 = lane >> 3, l8 = lane & 7;  // ldmatrix: this lane's matrix and row
   pdl_trigger();
   cta_copy(tb, tabs, T_ROW * 2);
   load_w(wbf + woff, nullptr, wt);
   pdl_wait();
-  float dw[4] = {0.f, 0.f, 0.f, 0.f};
-  float db = 0.f;
+  float gw[2][4][4];  // grad W [16 o][8 i] tiles of this warp's pixels
+  float2 gb[2][2];    // sums of dpre over the thread's even and odd pixels, channels 16 m + 8 e + g
+#pragma unroll
+  for (int m = 0; m < 2; ++m) {
+    gb[m][0] = gb[m][1] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int n = 0; n < 4; ++n) gw[m][n][0] = gw[m][n][1] = gw[m][n][2] = gw[m][n][3] = 0.f;
+  }
+  const uint32_t s0 = smem_addr(sm);
+  // ldmatrix row addresses of the lane.  A tiles (16 rows x 16 of K): matrices (rows 0-7 | 8-15) x (K 0-7 | 8-15);
+  // B tiles of one n-tile over K = 32, or of two n-tiles over K = 16
+  const int ar = (j8 & 1) * 8 + l8, ak = (j8 >> 1) * 16;
+  const uint32_t aZ = s0 + RB_Z + ar * RBZ + ak, aW = s0 + RB_W + ar * (WP * 2) + ak, aP = s0 + RB_P + ar * RBP + ak;
+  const uint32_t bI = s0 + 4 * T_RF + (16 * warp + l8) * RBZ + j8 * 16;  // RowI [ix][kyc], after RowF hi, lo
+  const uint32_t bF = s0 + ((j8 >> 1) * 8 + l8) * RBP + (j8 & 1) * 16;   // RowF [kyc][ix]
+  constexpr int ZPL = 2 * FC * RBZ, PPL = 2 * FC * RBP;                  // bytes of a plane
+  const int zr = tid & 63, zq = tid >> 6;                                // dU row and four ky this thread stages
+  const int p0 = 16 * warp;
   const int items = B * NIB;
   for (int it = blockIdx.x; it < items; it += gridDim.x) {
-    const int b = it / NIB, iyb = it % NIB, iy0 = iyb * RB;
-    const long long pix0 = (long long)iy0 * FN;
-    const long long gbase = (long long)b * FC * FNN + pix0;
-    load_planar(gs, dvp, b, pix0);
-    load_planar(vs, v, b, pix0);
-    if (dU) cta_copy(zs, dU + ((long long)b * NIB + iyb) * BLK, BLK * 8);
-    cp_wait_all();
-    __syncthreads();
+    const int b = it / NIB, iyb = it % NIB;
+    const long long gbase = (long long)b * FC * FNN + (long long)iyb * NP + p0 + 2 * t;
     if (dU) {
-      row_inverse(zs, tb, gs, true);
-      __syncthreads();
+      const float2* zb = dU + ((long long)b * NIB + iyb) * BLK + (4 * zq * FC + (zr & 31)) * RB + (zr >> 5);
+      float2 z[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) z[m] = __ldg(zb + m * FC * RB);
+      uint4 h, l;
+      split_pair(z[0].x, z[0].y, h.x, l.x);
+      split_pair(z[1].x, z[1].y, h.y, l.y);
+      split_pair(z[2].x, z[2].y, h.z, l.z);
+      split_pair(z[3].x, z[3].y, h.w, l.w);
+      *reinterpret_cast<uint4*>(sm + RB_Z + zr * RBZ + 16 * zq) = h;
+      *reinterpret_cast<uint4*>(sm + RB_Z + ZPL + zr * RBZ + 16 * zq) = l;
     }
-    if (act)
-      planar_pass(gs, gbase, [&](float4& x, long long gi) {
-        const float4 p = *reinterpret_cast<const float4*>(pre + gi);
-        const float2 a = pair_mul(make_float2(x.x, x.y), gelu_grad_f(make_float2(p.x, p.y)));
-        const float2 b = pair_mul(make_float2(x.z, x.w), gelu_grad_f(make_float2(p.z, p.w)));
-        x = make_float4(a.x, a.y, b.x, b.y);
-      });
+    cp_wait_all();  // (the tables, once)
     __syncthreads();
-    // dvp_out = W^T dpre: GEMM M = NP, N = FC (i), K = FC (o)
-    pixel_mix([&](int p, int o) { return gs[o * NPP + p]; }, wt,
-              [&](int p, int i, float val) { dvp_out[gbase + (long long)i * FNN + p] = val; });
-    {  // grad W += dpre v^T: GEMM M = FC (o), N = FC (i), K = NP; warp = one 16 x 8 tile
-      auto A = [&](int o, int p) { return gs[o * NPP + p]; };
-      auto Bv = [&](int p, int i) { return vs[i * NPP + p]; };
-      const int mt = warp & 1, nt = warp >> 1;
-#pragma unroll 4
-      for (int ks = 0; ks < NP / 16; ++ks) mma3(dw, load_a(A, 16 * mt, 16 * ks, g, t), load_b(Bv, 16 * ks, 8 * nt, g, t));
-      const int o = threadIdx.x >> 3;
-      for (int p = threadIdx.x & 7; p < NP; p += 8) db += gs[o * NPP + p];
+#pragma unroll
+    for (int r = 0; r < RB; ++r) {
+      const float* src = dvp + gbase + r * FN;
+      float d[2][2][4];  // [m: 16 channels][n: 8 pixels]: channels g, g + 8, pixels 2t, 2t + 1
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const float2 x = *reinterpret_cast<const float2*>(src + (long long)(16 * m + 8 * e + g) * FNN + 8 * n);
+            d[m][n][2 * e] = x.x;
+            d[m][n][2 * e + 1] = x.y;
+          }
+      if (dU) {
+        float s[2][2][4] = {};
+        uint32_t bh[2][4], bl[2][4];
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+          ldsm4(bh[n], bI + 8 * n * RBZ);
+          ldsm4(bl[n], bI + 8 * n * RBZ + 2 * T_RI);
+        }
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks) {
+            FragA a;
+            ldsm4(a.h, aZ + (FC * r + 16 * m) * RBZ + 32 * ks);
+            ldsm4(a.l, aZ + (FC * r + 16 * m) * RBZ + 32 * ks + ZPL);
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+              const uint32_t h2[2] = {bh[n][2 * ks], bh[n][2 * ks + 1]}, l2[2] = {bl[n][2 * ks], bl[n][2 * ks + 1]};
+              mma3t(s[m][n], a, h2, l2);
+            }
+          }
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) d[m][n][e] += s[m][n][e];
+      }
+      FragA dp[2];  // dpre as A fragments [16 o][16 pixels]
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            float2 x = make_float2(d[m][n][2 * e], d[m][n][2 * e + 1]);
+            const int c = 16 * m + 8 * e + g;
+            if (act)
+              x = pair_mul(x, gelu_grad_f(*reinterpret_cast<const float2*>(pre + gbase + r * FN + (long long)c * FNN + 8 * n)));
+            gb[m][e] = pair_add(gb[m][e], x);
+            split_pair(x.x, x.y, dp[m].h[2 * n + e], dp[m].l[2 * n + e]);
+            unsigned char* o = sm + RB_P + (FC * r + c) * RBP + (p0 + 8 * n + 2 * t) * 2;
+            *reinterpret_cast<uint32_t*>(o) = dp[m].h[2 * n + e];
+            *reinterpret_cast<uint32_t*>(o + PPL) = dp[m].l[2 * n + e];
+          }
+      // grad W += dpre v^T over the 16 pixels
+#pragma unroll
+      for (int n = 0; n < 4; ++n) {
+        const float* vs = v + gbase + r * FN + (long long)(8 * n + g) * FNN;
+        const float2 x0 = *reinterpret_cast<const float2*>(vs), x1 = *reinterpret_cast<const float2*>(vs + 8);
+        FragB bv;
+        split_pair(x0.x, x0.y, bv.h[0], bv.l[0]);
+        split_pair(x1.x, x1.y, bv.h[1], bv.l[1]);
+        mma3(gw[0][n], dp[0], bv);
+        mma3(gw[1][n], dp[1], bv);
+      }
+      // dvp_out [i][16 pixels] = W^T dpre, K = o
+      float w[2][2][4] = {};
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) {
+        uint32_t aw[2][4];
+        ldsm4(aw[0], aW + 32 * ks);
+        ldsm4(aw[1], aW + 16 * (WP * 2) + 32 * ks);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+          const uint32_t h2[2] = {transpose8(dp[ks].h[2 * n]), transpose8(dp[ks].h[2 * n + 1])};
+          const uint32_t l2[2] = {transpose8(dp[ks].l[2 * n]), transpose8(dp[ks].l[2 * n + 1])};
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            mma16816(w[m][n], aw[m], h2);
+            mma16816(w[m][n], aw[m], l2);
+          }
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            *reinterpret_cast<float2*>(dvp_out + gbase + r * FN + (long long)(16 * m + 8 * e + g) * FNN + 8 * n) =
+                make_float2(w[m][n][2 * e], w[m][n][2 * e + 1]);
     }
-    row_forward(gs, tb, zs);
+    __syncthreads();
+    // dT [16 rr][16 kyc] of this warp = RowF(dpre), K = the 128 pixels
+    float f[2][4] = {};
+    const int mt = warp & 3, nh = warp >> 2;
+#pragma unroll 2
+    for (int k0 = 0; k0 < FN; k0 += 16) {
+      FragA a;
+      ldsm4(a.h, aP + 16 * mt * RBP + 2 * k0);
+      ldsm4(a.l, aP + 16 * mt * RBP + 2 * k0 + PPL);
+      uint32_t bh[4], bl[4];
+      ldsm4(bh, bF + 16 * nh * RBP + 2 * k0);
+      ldsm4(bl, bF + 16 * nh * RBP + 2 * k0 + 2 * T_RF);
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        const uint32_t h2[2] = {bh[2 * n], bh[2 * n + 1]}, l2[2] = {bl[2 * n], bl[2 * n + 1]};
+        mma3t(f[n], a, h2, l2);
+      }
+    }
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int rr = 16 * mt + g + 8 * e, ky = 8 * nh + 4 * n + t;
+        stage[(ky * FC + (rr & 31)) * RB + (rr >> 5)] = make_float2(f[n][2 * e], f[n][2 * e + 1]);
+      }
     __syncthreads();
     float4* dst = reinterpret_cast<float4*>(dT + ((long long)b * NIB + iyb) * BLK);
-    for (int i = threadIdx.x; i < BLK / 2; i += NTH) dst[i] = reinterpret_cast<float4*>(zs)[i];
-    __syncthreads();
+    for (int i = tid; i < BLK / 2; i += NTH) dst[i] = reinterpret_cast<float4*>(stage)[i];
   }
-  float* pp = part + (long long)blockIdx.x * PART_W;
-  {
-    const int mt = warp & 1, nt = warp >> 1;
+  __syncthreads();
+  // the eight warps' partials, summed in warp order
+  float* red = reinterpret_cast<float*>(sm + RB_Z) + warp * PART_W;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) pp[(16 * mt + g + (e >> 1) * 8) * FC + 8 * nt + 2 * t + (e & 1)] = dw[e];
+  for (int m = 0; m < 2; ++m) {
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) red[(16 * m + g + 8 * (e >> 1)) * FC + 8 * n + 2 * t + (e & 1)] = gw[m][n][e];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      float s = gb[m][e].x + gb[m][e].y;
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      if (t == 0) red[FC * FC + 16 * m + 8 * e + g] = s;
+    }
   }
-  db += __shfl_xor_sync(0xffffffffu, db, 1);
-  db += __shfl_xor_sync(0xffffffffu, db, 2);
-  db += __shfl_xor_sync(0xffffffffu, db, 4);
-  if ((threadIdx.x & 7) == 0) pp[FC * FC + (threadIdx.x >> 3)] = db;
+  __syncthreads();
+  for (int i = tid; i < PART_W; i += NTH) {
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < NTH / 32; ++w) s += reinterpret_cast<const float*>(sm + RB_Z)[w * PART_W + i];
+    part[(long long)blockIdx.x * PART_W + i] = s;
+  }
 }
 
 // Projection backward, persistent over image rows (128 pixels): recomputes z = P1 v4 + c1, dz = (P2^T dout) GELU'(z);
@@ -1022,14 +1181,6 @@ constexpr int PBV = 80;            // bytes of a pixel's 32 channels in a plane 
 constexpr int PBD = 2 * (FN + 8);  // bytes of a hidden unit's 128 pixels in a plane of dz
 constexpr int PB_V = 0, PB_D = PB_V + 2 * FN * PBV, PB_P1T = PB_D + 2 * FH * PBD, PB_DS = PB_P1T + FC * P1TP * 2,
               SM_PBWD = PB_DS + 2 * FN * 4;
-__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
 __global__ void __launch_bounds__(NTH, 2) fno_proj_bwd(const float* __restrict__ v4, const float* __restrict__ dout,
                                                        const __nv_bfloat16* __restrict__ wbf,
                                                        const float* __restrict__ pm, int B,
