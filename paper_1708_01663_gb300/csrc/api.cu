@@ -81,9 +81,11 @@ struct Call {
     return CISOR_OK;
   }
   // *use: an input where kernels can read it: src itself, or its copy in buf.  out, out2: what they write meanwhile.
+  // mask: low address bits that must be clear (15 for kernels that read two values at a time)
   cisor_status operand(const float2** use, const void* src, float2* buf, size_t bytes, const void* out = nullptr,
-                       size_t out_bytes = 0, const void* out2 = nullptr) {
-    const bool direct = in_place(c, src) && !overlap(src, bytes, out, out_bytes) && !overlap(src, bytes, out2, out_bytes);
+                       size_t out_bytes = 0, const void* out2 = nullptr, uintptr_t mask = 7) {
+    const bool direct = in_place(c, src) && !((uintptr_t)src & mask) && !overlap(src, bytes, out, out_bytes) &&
+                        !overlap(src, bytes, out2, out_bytes);
     *use = direct ? (const float2*)src : buf;
     return direct ? CISOR_OK : in(buf, src, bytes);
   }
@@ -349,7 +351,7 @@ cisor_status cisor_create(cisor_ctx** out, const cisor_geometry* g, void* stream
   if (conv3_ok(d, P)) ALLOC(c->gplane, sizeof(float2) * conv3_ghat_elems(P));
   ALLOC(c->tw, sizeof(float2) * P);
   ALLOC(c->twst, sizeof(float2) * 2 * 512);
-  ALLOC(c->H, (size_t)c->M * c->Nf * sizeof(float2));
+  ALLOC(c->H, sense_h_bytes(c));
   ALLOC(c->u_in, TN);
   ALLOC(c->R, (size_t)c->T * c->ncomp * c->rtstride * sizeof(float2));
   ALLOC(c->r, TN);
@@ -374,7 +376,7 @@ cisor_status cisor_create(cisor_ctx** out, const cisor_geometry* g, void* stream
   {
     int ks = c->ksplit;
     if (sense_tc_ok(c)) {  // tensor-core sensing: the transposed matrix, the timeout flag, its split-K partials
-      ALLOC(c->Ht, (size_t)c->M * c->Nf * sizeof(float2));
+      ALLOC(c->Ht, sense_ht_bytes(c));
       cudaError_t e = cudaHostAlloc((void**)&c->h_tc_err, sizeof(int), cudaHostAllocMapped);
       if (e == cudaSuccess) {
         *c->h_tc_err = 0;
@@ -457,7 +459,16 @@ cisor_status cisor_sensing_matrix(cisor_ctx* c, void* out) {
   }
   Call call(c);
   CISOR_TRY(call.enter());
-  CISOR_TRY(call.out(out, c->H, sizeof(float2) * (size_t)c->M * c->Nf));
+  const size_t row = sizeof(float2) * (size_t)c->Nf;
+  if (in_place(c, out)) {
+    CISOR_TRY(sense_h_rows(c, 0, c->M, (float2*)out));
+    return call.leave();
+  }
+  for (long long m = 0; m < c->M; m += c->T) {  // T rows at a time through the solver's workspace
+    const long long k = c->M - m < c->T ? c->M - m : c->T;
+    CISOR_TRY(sense_h_rows(c, m, k, c->tv));
+    CISOR_TRY(call.out((char*)out + m * row, c->tv, k * row));
+  }
   return call.leave();
 }
 
@@ -565,8 +576,8 @@ cisor_status cisor_sense(cisor_ctx* c, const void* f, const void* u, void* Z_out
   Call call(c);
   CISOR_TRY(call.enter());
   const float2 *fd, *ud;  // (the GEMM has read both before its reduction writes Z)
-  CISOR_TRY(call.operand(&fd, f, c->f, sizeof(float2) * c->N));
-  CISOR_TRY(call.operand(&ud, u, c->s, sizeof(float2) * (size_t)c->T * c->Nf));
+  CISOR_TRY(call.operand(&fd, f, c->f, sizeof(float2) * c->N, nullptr, 0, nullptr, 15));
+  CISOR_TRY(call.operand(&ud, u, c->s, sizeof(float2) * (size_t)c->T * c->Nf, nullptr, 0, nullptr, 15));
   const bool direct = in_place(c, Z_out);
   CISOR_TRY(sense_forward(c, fd, ud, direct ? (float2*)Z_out : c->Y, c->T));
   if (!direct) CISOR_TRY(call.out(Z_out, c->Y, sizeof(float2) * (size_t)c->T * c->M));
@@ -584,7 +595,7 @@ cisor_status cisor_sense_adjoint(cisor_ctx* c, const void* f, const void* w, voi
   const size_t vb = sizeof(float2) * (size_t)c->T * c->Nf;
   const float2 *fd, *wd;
   CISOR_TRY(call.operand(&fd, f, c->f, sizeof(float2) * c->N, z_out, vb, b_out));
-  CISOR_TRY(call.operand(&wd, w, c->w, sizeof(float2) * (size_t)c->T * c->M, z_out, vb, b_out));
+  CISOR_TRY(call.operand(&wd, w, c->w, sizeof(float2) * (size_t)c->T * c->M, z_out, vb, b_out, 15));
   const bool apart = !overlap(z_out, vb, b_out, vb);
   const bool zdir = apart && in_place(c, z_out), bdir = apart && in_place(c, b_out);
   float2* b = bdir ? (float2*)b_out : (b_out ? c->b : nullptr);

@@ -15,16 +15,37 @@
 //   adjoint  z_t[n] = sum_m conj(H[m][n]) w_t[m] (H^H w, Eq. 13), read from the
 //            transposed copy Ht[n][m] so that both GEMMs stream K-major rows:
 //            rows 2t = (Re w, Im w), 2t + 1 = (Im w, -Re w) per m
-// A CTA owns 128 rows of the big operand (receivers forward, field entries
-// adjoint) and 2T (rounded to 16) accumulator columns in tensor memory; it
-// streams 32 floats of K per chunk: each thread loads 4 x 16 bytes of the big
-// operand for the next chunk into registers while the current chunk's MMAs
-// run, splits them and stores them as core-matrix rows (8 rows x 16 bytes, K
-// groups 144 bytes apart so that the 8 lanes of a 16-byte store phase hit
-// distinct banks).  The forward pass splits K over CTAs (partials [split][T][M]
-// summed by sense_reduce_kernel, in a fixed order); the adjoint CTA covers all
-// of K (2M) and writes z and conj(f) z.  Every wait on the MMAs is bounded (a
-// timeout sets the context's error flag, read by the host after the call).
+// An accumulator tile is 128 rows of the big operand (receivers forward, field
+// entries adjoint) by 2T columns (rounded up to NB) in tensor memory, and K is
+// streamed in chunks of 32 floats.  The forward pass splits K into slabs
+// (partials [split][T][M] summed by sense_reduce_kernel, in a fixed order); an
+// adjoint tile covers all of K (2M) and writes z and conj(f) z.
+//
+// Up to 96 transmitters (NB <= 192) H and Ht are stored as those tiles: 128 rows
+// by 32 floats, contiguous, in the order in which a CTA streams them (tile_off), so
+// that a chunk is one 16 KB bulk copy by one thread; the copies alone run at 7.3
+// TB/s.  One warp-specialised CTA per SM runs over the tiles (sense_ws_kernel): a
+// thread keeps SENSE_STAGES bulk copies of the big operand in flight, converter
+// warps split each chunk into hi / lo planes in TENSOR MEMORY, builder warps write
+// the small operand's planes to shared memory, two threads issue the MMAs (A from
+// tensor memory, B from shared memory) and the remaining warps add finished chunks
+// into FP32 registers; several buffers of everything behind the load ring let all
+// roles work on different chunks at once.  A in tensor memory is what makes the
+// shared-memory pipe suffice: per 16 KB chunk it carries the copy, one read, the
+// small operand's write and its reads by the MMAs (93 KB at NB = 96 against 140 KB
+// with both planes of A there).
+// Measured at 48 transmitters, 1024 receivers, 64^3 (H and Ht of 2.1 GB): forward
+// 1.15 -> 0.67 ms, adjoint 0.93 -> 0.58 ms against the kernel below on row-major
+// matrices, which does all roles in every thread; 64 transmitters, 256 receivers,
+// 256^2: 0.136 -> 0.078, 0.092 -> 0.085; 81, 36, 32^3 vectorial: 0.108 -> 0.097,
+// 0.096 -> 0.068; 8, 360, 128^2: 0.044 -> 0.024, 0.037 -> 0.017; 8, 32, 64^2: 0.017 -> 0.015,
+// 0.008 -> 0.007 (all launches; slower only with two receivers and many
+// transmitters, whose chunks are mostly padding: 48, 2, 256^2 adjoint 20 -> 24 us).  What bounds it: the hand-overs between the roles
+// (below); the MMAs keep the tensor pipe about half of the time at NB = 96, the
+// copies the memory for 45%.  More than 96 transmitters leave no room for two
+// accumulators and A in tensor memory and take the kernel below (sense_tc_kernel).
+// Every wait is bounded (a timeout sets the context's error flag, read by the host
+// after the call).
 #include "common.cuh"
 #include "tc5.cuh"
 
@@ -45,6 +66,15 @@ constexpr long long S_MAX = 256;  // at most this many splits (partials T x M x 
 __host__ __device__ constexpr int soff(int row, int k) {
   return (row >> 3) * SSBO + (k >> 2) * SLBO + (row & 7) * 16 + (k & 3) * 4;
 }
+// float offset of (row, k) in a tiled [rows][Kp] matrix: tiles of 128 rows, chunks of SK floats within a tile (its
+// rows' 128 bytes one after another), 16-byte piece j of row r at j ^ (r % 8), so that 8 threads reading the same
+// piece of 8 rows from shared memory hit distinct banks.  Kp: the row length rounded up to SK (zeros behind it).
+__host__ __device__ __forceinline__ long long tile_kp(long long width) { return (width + SK - 1) / SK * SK; }
+__host__ __device__ __forceinline__ long long tile_off(long long row, long long k, long long rows, long long Kp) {
+  const long long r0 = row & ~127ll, R = rows - r0 < 128 ? rows - r0 : 128;
+  const int r = (int)(row - r0), j = (int)(k & (SK - 1)) >> 2;
+  return r0 * Kp + (k / SK) * (R * SK) + r * SK + ((j ^ (r & 7)) << 2) + (k & 3);
+}
 __device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
 __device__ __forceinline__ long long wrap(long long j, long long NP) {
   while (j >= NP) j -= NP;
@@ -56,7 +86,7 @@ int sense_tc_cols(int ntx) {
   const int need = 2 * ntx;
   return need <= 32 ? 32 : need <= 64 ? 64 : need <= 96 ? 96 : need <= 128 ? 128 : need <= 192 ? 192 : 256;
 }
-int sense_tc_smem(int ntx) { return 2 * SPA + 2 * (sense_tc_cols(ntx) / 8) * SSBO; }
+constexpr int WS_NB = 192;  // most accumulator columns of the warp-specialised kernel: 2 x 192 and A's 128 fill the 512
 
 // ADJ = 0: A = H [rows = M][lda = 2 Nf], K range [ks KS, ks KS + KS) of 2 Nf, small operand from f and u [T][Nf];
 //          out0 = partials [(ks T + t) M + m].
@@ -214,6 +244,307 @@ __global__ void __launch_bounds__(STH, NB > 128 ? 1 : 2) sense_tc_kernel(const f
   if (warp == 0) tmem_dealloc(tmem, ncol);
 }
 
+// ------------------------------------------------------------------ warp-specialised kernel, NB <= 192
+// Up to 128 columns: warps 0-7 are A converters, two groups of four on alternate chunks (thread = tile row =
+// tensor-memory lane), 8-15 accumulate (lane quarter w % 4, columns halved), 16-23 build B, two groups on alternate
+// chunks.  192 columns: 4 converters, 12 accumulators (thirds of the columns: 96 a thread would spill), 4 builders.
+// Then the producer of the bulk copies and two MMA issuers.
+// Chunk n of the CTA's sequence over all its tiles uses load stage n % SENSE_STAGES, operand buffer n % DEP (A in
+// tensor memory, B in shared memory) and accumulator n % ND.  An MMA issuer waits once a chunk: `ready` collects the
+// converters', the builders' and the accumulators' arrivals (the last for the chunk ND before, whose accumulator this
+// one reuses).  A completed barrier still costs its waiter 200 to 350 cycles and a commit 300, against about 650 for
+// the chunk's MMAs at NB = 96; that is why the roles run up to DEP chunks apart and why two threads issue, each
+// waiting while the other's MMAs run.  Forward / adjoint at 48 transmitters, 64^3: 0.99 / 0.80 ms with one group of
+// builders and one issuer, 0.73 / 0.64 with two groups, 0.67 / 0.58 with two issuers.
+// operand buffers and accumulators (at most as many): what 512 columns of tensor memory hold.  An even number of
+// buffers: then a buffer's chunks belong to one group of converters and of builders and to one issuer, so that nobody
+// tests a barrier that is still a phase behind the one it waits for.
+__host__ __device__ constexpr int ws_dep(int nb) { return nb <= 96 ? 4 : 2; }
+__host__ __device__ constexpr int ws_nd(int nb) { return nb <= 64 ? 4 : 2; }
+__host__ __device__ constexpr int ws_groups(int nb) { return nb <= 128 ? 2 : 1; }  // of four builder warps, and of four converters
+constexpr int WS_ISS = 2;  // MMA issuers, on alternate chunks
+__host__ __device__ constexpr int ws_threads(int nb) { return (17 + WS_ISS + 4 * ws_groups(nb)) * 32; }
+constexpr int SENSE_STAGES = 6;
+constexpr int WS_A = 128 * SK * 4;  // bytes of a chunk of A
+constexpr int ws_smem(int nb) { return 1024 + SENSE_STAGES * WS_A + ws_dep(nb) * 2 * (nb / 8) * SSBO; }
+
+struct WsBars {
+  uint64_t full[SENSE_STAGES], empty[SENSE_STAGES], ready[4], done[4];
+};
+
+template <int ADJ, int NB>
+__global__ void __launch_bounds__(ws_threads(NB), 1) sense_ws_kernel(const float* __restrict__ A, long long rows, int rtiles,
+                                                            int nitems, long long K, long long KS,
+                                                            const float2* __restrict__ src, long long lds,
+                                                            const float2* __restrict__ f, long long NP, int T, int M,
+                                                            long long Nf, float2* __restrict__ out0,
+                                                            float2* __restrict__ out1, int* __restrict__ err) {
+  extern __shared__ unsigned char smraw[];
+  __shared__ __align__(8) WsBars bar;
+  __shared__ uint32_t tslot;
+  __shared__ volatile int failed;
+  unsigned char* sm = smraw + ((1024 - (smem_addr(smraw) & 1023)) & 1023);
+  constexpr int SPB = (NB / 8) * SSBO;   // bytes of a plane of B
+  constexpr int IPT = NB / 32;           // (transmitter, two complex columns) pieces per building thread
+  constexpr int DEP = ws_dep(NB), ND = ws_nd(NB), GB = ws_groups(NB), TH = ws_threads(NB);
+  constexpr int NH = NB / (4 - GB);      // accumulator columns per accumulating thread
+  constexpr uint32_t ACOL = ND * NB;     // tensor memory: ND accumulators, then DEP x (hi, lo) of A
+  static_assert(ND * NB + 64 * DEP <= 512 && ND <= DEP, "tensor memory columns");
+  static_assert(DEP % 2 == 0 && SENSE_STAGES % 2 == 0, "a buffer or stage belongs to one group, one issuer");
+  unsigned char* sb = sm + SENSE_STAGES * WS_A;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid * 16; i < 2 * DEP * SPB; i += TH * 16) *reinterpret_cast<uint4*>(sb + i) = make_uint4(0, 0, 0, 0);
+  if (tid == 0) {
+    failed = 0;
+    for (int i = 0; i < SENSE_STAGES; ++i) {
+      mbar_init(&bar.full[i]);
+      mbar_init(&bar.empty[i], 4);
+    }
+    for (int i = 0; i < DEP; ++i) {
+      mbar_init(&bar.ready[i], 4 + 4 + 4 * (4 - GB));
+      mbar_init(&bar.done[i]);
+    }
+  }
+  if (warp == 0) tmem_alloc(&tslot, 512);
+  fence_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tslot;
+  // false (and everyone told) if a wait gave up, here or in another role
+  auto wait = [&](uint64_t* b, uint32_t use) {
+    for (int it = 0; it < S_WAIT; ++it) {
+      if (mbar_wait(b, use & 1, 1)) return true;
+      if (failed) return false;
+    }
+    failed = 1;
+    *reinterpret_cast<volatile int*>(err) = 1;  // mapped host memory: a plain store
+    return false;
+  };
+  auto wait_warp = [&](uint64_t* b, uint32_t use) { return (bool)__all_sync(0xffffffffu, wait(b, use)); };
+  auto arrive = [&](uint64_t* b) {  // one arrival per warp, after all of its lanes
+    __syncwarp();
+    if (lane == 0) mbar_arrive(b);
+  };
+  // this CTA's tiles: row tile, first and last K of the slab, chunks
+  struct Item {
+    long long row0, kb, ke;
+    int split, nch;
+  };
+  auto item = [&](int it) {
+    Item r;
+    r.split = ADJ ? 0 : it / rtiles;
+    r.row0 = (long long)(ADJ ? it : it % rtiles) * 128;
+    r.kb = r.split * KS;
+    r.ke = r.kb + KS < K ? r.kb + KS : K;
+    r.nch = (int)((r.ke - r.kb + SK - 1) / SK);
+    return r;
+  };
+  uint32_t total = 0;  // chunks of this CTA
+  for (int it = blockIdx.x; it < nitems; it += gridDim.x) total += item(it).nch;
+  if (warp < 4 * GB) {  // ---- converters: hi / lo planes of a chunk of A into tensor memory
+    const int row = 32 * (warp & 3) + lane;
+    const uint32_t ta = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + ACOL;
+    for (uint32_t n = warp >> 2; n < total; n += GB) {
+      const uint32_t s = n % SENSE_STAGES, buf = n % DEP, k = n / DEP;
+      if (!wait_warp(&bar.full[s], n / SENSE_STAGES)) break;
+      const unsigned char* p = sm + s * WS_A + row * 128;  // (tile_off)
+      uint32_t h[32], l[32];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float4 x = *reinterpret_cast<const float4*>(p + ((j ^ (row & 7)) << 4));
+        const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float hi = tf32_hi(v[e]);
+          h[4 * j + e] = __float_as_uint(hi);
+          l[4 * j + e] = __float_as_uint(v[e] - hi);
+        }
+      }
+      if (k >= 1 && !wait_warp(&bar.done[buf], k - 1)) break;  // the planes' last reader
+      tc_fence_after();
+      tmem_st32(ta + 64 * buf, h);
+      tmem_st32(ta + 64 * buf + 32, l);
+      arrive(&bar.empty[s]);  // here, where the stores needed all values, not behind the loads' issue: the next copy into
+                              // the stage overtook loads still on their way (wrong values in 40% of some runs)
+      tmem_wait_st();
+      tc_fence_before();
+      arrive(&bar.ready[buf]);
+    }
+  } else if (warp < 16) {  // ---- accumulation
+    const int q = warp & 3, part = (warp - 4 * GB) >> 2;
+    const uint32_t td = tmem + ((uint32_t)(32 * q) << 16) + part * NH;
+    for (int i = 0; i < ND; ++i) arrive(&bar.ready[i]);  // the first chunks' accumulators are free
+    uint32_t n = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
+      const Item r = item(it);
+      float acc[NH];
+#pragma unroll
+      for (int j = 0; j < NH; ++j) acc[j] = 0.f;
+      for (int ch = 0; ch < r.nch; ++ch, ++n) {
+        if (!(ok = wait_warp(&bar.done[n % DEP], n / DEP))) break;
+        tc_fence_after();
+#pragma unroll
+        for (int c0 = 0; c0 < NH; c0 += 8) {
+          float d[8];
+          tmem_ld8(td + n % ND * NB + c0, d);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[c0 + j] += d[j];
+        }
+        tc_fence_before();
+        arrive(&bar.ready[(n + ND) % DEP]);
+      }
+      const long long row = r.row0 + 32 * q + lane;
+      if (!ok || row >= rows) continue;
+#pragma unroll
+      for (int c0 = 0; c0 < NH; c0 += 2) {
+        const int t = (part * NH + c0) / 2;
+        if (t >= T) break;
+        const float2 v = make_float2(acc[c0], acc[c0 + 1]);
+        if (!ADJ) {
+          out0[((long long)r.split * T + t) * M + row] = v;
+        } else {
+          out0[(long long)t * Nf + row] = v;
+          if (out1) out1[(long long)t * Nf + row] = c_cjmul(__ldg(f + wrap(row, NP)), v);
+        }
+      }
+    }
+  } else if (warp < 16 + 4 * GB) {  // ---- builders: hi / lo planes of the small operand into shared memory
+    // the values of a group's next two chunks are on their way from global memory while a third is staged; a thread has
+    // the columns 2 c2, 2 c2 + 1 (16 bytes; src, f and their rows are 16-byte aligned) of transmitters t0 + 16 i
+    const int bt = (tid - 16 * 32) & 127, group = (warp - 16) >> 2, c2 = bt & 7, t0 = bt >> 3;
+    float4 rb[2][IPT], rf[2];
+    const long long step = 16 * lds;
+    // the group's next chunk to fetch: tile, chunk in it, where its values lie and K left from this thread's columns on
+    int fit = blockIdx.x, fch = 0, fn = 0, left = 0;
+    const float2 *fp = nullptr, *ff = nullptr;
+    auto enter = [&]() {
+      const Item r = item(fit);
+      fn = r.nch;
+      left = (int)(r.ke - r.kb) - 4 * c2;
+      fp = src + (long long)t0 * lds + r.kb / 2 + 2 * c2;
+      if (!ADJ) ff = f + wrap(r.kb / 2 + 2 * c2, NP);
+    };
+    auto advance = [&](int by) {  // by chunks, over tile ends
+      fch += by;
+      left -= by * SK;
+      fp += by * (SK / 2);
+      if (!ADJ) {
+        ff += by * (SK / 2);
+        while (ff >= f + NP) ff -= NP;
+      }
+      while (fit < nitems && fch >= fn) {
+        fch -= fn;
+        fit += gridDim.x;
+        if (fit >= nitems) break;
+        enter();
+        if (fch) {
+          left -= fch * SK;
+          fp += fch * (SK / 2);
+          if (!ADJ) {
+            ff += fch * (SK / 2);
+            while (ff >= f + NP) ff -= NP;
+          }
+        }
+      }
+    };
+    uint32_t n = group;
+    auto fetch = [&](float4 (&x)[IPT], float4& fx) {
+      if (fit >= nitems) return;
+      const bool in = left > 0;
+#pragma unroll
+      for (int i = 0; i < IPT; ++i)
+        x[i] = in && t0 + 16 * i < T ? __ldg(reinterpret_cast<const float4*>(fp + i * step)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      if (!ADJ) fx = in ? __ldg(reinterpret_cast<const float4*>(ff)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      advance(GB);
+    };
+    // stages chunk n from x, then refills x for the group's chunk after the next; false once a wait gave up
+    auto build = [&](float4 (&x)[IPT], float4& fx) {
+      const uint32_t buf = n % DEP, k = n / DEP;
+      if (k >= 1 && !wait_warp(&bar.done[buf], k - 1)) return false;
+      unsigned char* d = sb + buf * 2 * SPB;
+#pragma unroll
+      for (int i = 0; i < IPT; ++i) {
+        const int t = t0 + 16 * i;
+        if (t < T) {
+          float2 v = make_float2(x[i].x, x[i].y), u = make_float2(x[i].z, x[i].w);
+          if (!ADJ) {
+            v = c_mul(make_float2(fx.x, fx.y), v);
+            u = c_mul(make_float2(fx.z, fx.w), u);
+          }
+          const float hx = tf32_hi(v.x), hy = tf32_hi(v.y), gx = tf32_hi(u.x), gy = tf32_hi(u.y);
+          const float lx = v.x - hx, ly = v.y - hy, kx = u.x - gx, ky = u.y - gy;
+          const int o0 = soff(2 * t, 4 * c2), o1 = soff(2 * t + 1, 4 * c2);
+          *reinterpret_cast<float4*>(d + o0) = ADJ ? make_float4(hx, hy, gx, gy) : make_float4(hx, -hy, gx, -gy);
+          *reinterpret_cast<float4*>(d + SPB + o0) = ADJ ? make_float4(lx, ly, kx, ky) : make_float4(lx, -ly, kx, -ky);
+          *reinterpret_cast<float4*>(d + o1) = ADJ ? make_float4(hy, -hx, gy, -gx) : make_float4(hy, hx, gy, gx);
+          *reinterpret_cast<float4*>(d + SPB + o1) = ADJ ? make_float4(ly, -lx, ky, -kx) : make_float4(ly, lx, ky, kx);
+        }
+      }
+      fence_async_smem();
+      arrive(&bar.ready[buf]);
+      fetch(x, fx);
+      n += GB;
+      return true;
+    };
+    enter();
+    if (group) advance(group);
+    fetch(rb[0], rf[0]);
+    fetch(rb[1], rf[1]);
+    while (n < total) {
+      if (!build(rb[0], rf[0])) break;
+      if (n < total && !build(rb[1], rf[1])) break;
+    }
+  } else if (warp == 16 + 4 * GB) {  // ---- producer
+    if (lane == 0) {
+      const long long Kp = tile_kp(K);
+      uint32_t n = 0;
+      bool ok = true;
+      for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
+        const Item r = item(it);
+        const int R = rows - r.row0 < 128 ? (int)(rows - r.row0) : 128;  // (rows past the last keep old values)
+        const float* p = A + r.row0 * Kp + r.kb / SK * (R * SK);
+        for (int ch = 0; ch < r.nch; ++ch, ++n, p += R * SK) {
+          const uint32_t s = n % SENSE_STAGES;
+          if (n >= SENSE_STAGES && !(ok = wait(&bar.empty[s], n / SENSE_STAGES - 1))) break;
+          mbar_expect(&bar.full[s], R * SK * 4);
+          bulk_load(sm + s * WS_A, p, R * SK * 4, &bar.full[s]);
+        }
+      }
+      // the loads still in flight land before the CTA's shared memory goes
+      for (uint32_t m = n > SENSE_STAGES ? n - SENSE_STAGES : 0; m < n; ++m)
+        (void)mbar_wait(&bar.full[m % SENSE_STAGES], (m / SENSE_STAGES) & 1, S_WAIT);
+    }
+    __syncwarp();
+  } else {  // ---- MMA issuer
+    if (lane == 0) {
+      const uint32_t id = tc_idesc_tf32(128, NB), b0 = smem_addr(sb);
+      uint32_t n = warp - (17 + 4 * GB);
+      for (; n < total; n += WS_ISS) {
+        const uint32_t buf = n % DEP;
+        if (!wait(&bar.ready[buf], n / DEP)) break;
+        tc_fence_after();
+        const uint32_t d = tmem + n % ND * NB, a = tmem + ACOL + 64 * buf, b = b0 + buf * 2 * SPB;
+#pragma unroll
+        for (int ks = 0; ks < SK / 8; ++ks) {
+          const uint64_t bh = tc_desc(b + ks * 2 * SLBO, SLBO, SSBO), bl = tc_desc(b + SPB + ks * 2 * SLBO, SLBO, SSBO);
+          tc_mma_tf32_ts(d, a + 8 * ks, bh, id, ks > 0 ? 1u : 0u);
+          tc_mma_tf32_ts(d, a + 32 + 8 * ks, bh, id, 1u);
+          tc_mma_tf32_ts(d, a + 8 * ks, bl, id, 1u);
+        }
+        tc_commit(&bar.done[buf]);
+      }
+      // the MMAs still in flight end before the CTA's tensor memory goes
+      if (n >= WS_ISS) (void)mbar_wait(&bar.done[(n - WS_ISS) % DEP], ((n - WS_ISS) / DEP) & 1, S_WAIT);
+    }
+    __syncwarp();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
 // Ht[n][m] = H[m][n], 32 x 32 complex tiles through shared memory
 __global__ void __launch_bounds__(256) sense_transpose_kernel(const float2* __restrict__ H, int M, long long Nf,
                                                               float2* __restrict__ Ht) {
@@ -234,45 +565,90 @@ __global__ void __launch_bounds__(256) sense_transpose_kernel(const float2* __re
   }
 }
 
+// row-major H [rows][width floats] into tiles, and back; a thread moves 16 bytes (zeros behind the row's end)
+__global__ void __launch_bounds__(256) sense_tile_kernel(const float* __restrict__ in, long long rows, long long width,
+                                                         float* __restrict__ out) {
+  const long long Kp = tile_kp(width), k = 4 * ((long long)blockIdx.x * 256 + threadIdx.x);
+  if (k >= Kp) return;
+  for (long long row = blockIdx.y; row < rows; row += gridDim.y)
+    *reinterpret_cast<float4*>(out + tile_off(row, k, rows, Kp)) =
+        k < width ? *reinterpret_cast<const float4*>(in + row * width + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+__global__ void __launch_bounds__(256) sense_untile_kernel(const float* __restrict__ in, long long rows, long long width,
+                                                           long long row0, long long nrows, float2* __restrict__ out) {
+  const long long Kp = tile_kp(width), k = 2 * ((long long)blockIdx.x * 256 + threadIdx.x);
+  if (k >= width) return;
+  for (long long i = blockIdx.y; i < nrows; i += gridDim.y)
+    out[(i * width + k) / 2] = *reinterpret_cast<const float2*>(in + tile_off(row0 + i, k, rows, Kp));
+}
+// tiled Ht[n][m] = H[m][n] from tiled H, 32 x 32 complex blocks through shared memory
+__global__ void __launch_bounds__(256) sense_tile_transpose_kernel(const float* __restrict__ H, int M, long long Nf,
+                                                                   float* __restrict__ Ht) {
+  __shared__ float2 tile[32][33];
+  const long long n0 = (long long)blockIdx.x * 32, Kh = tile_kp(2 * Nf), Kt = tile_kp(2 * (long long)M);
+  const int m0 = blockIdx.y * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int i = ty; i < 32; i += 8) {
+    const int m = m0 + i;
+    const long long n = n0 + tx;
+    tile[i][tx] = m < M && n < Nf ? *reinterpret_cast<const float2*>(H + tile_off(m, 2 * n, M, Kh)) : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  for (int i = ty; i < 32; i += 8) {
+    const long long n = n0 + i;
+    const int m = m0 + tx;
+    if (2 * m < Kt && n < Nf) *reinterpret_cast<float2*>(Ht + tile_off(n, 2 * (long long)m, Nf, Kt)) = tile[tx][i];
+  }
+}
+
 // ------------------------------------------------------------------ host side
 bool sense_tc_ok(const cisor_ctx* c) {
   // 16-byte rows of H and Ht (2 Nf and 2 M floats), 2T accumulator columns <= 256
   return c->T <= 128 && c->Nf % 2 == 0 && c->M % 2 == 0;
 }
+bool sense_tiled(const cisor_ctx* c) { return sense_tc_ok(c) && sense_tc_cols(c->T) <= WS_NB; }
+size_t sense_h_bytes(const cisor_ctx* c) {
+  return sense_tiled(c) ? sizeof(float) * (size_t)(c->M * tile_kp(2 * c->Nf)) : sizeof(float2) * (size_t)c->M * c->Nf;
+}
+size_t sense_ht_bytes(const cisor_ctx* c) {
+  return sense_tiled(c) ? sizeof(float) * (size_t)(c->Nf * tile_kp(2 * (long long)c->M)) : sizeof(float2) * (size_t)c->M * c->Nf;
+}
 
-// the kernel instance for nb accumulator columns (sense_tc_cols)
+// the warp-specialised kernel for nb <= 192 accumulator columns (sense_tc_cols)
 template <int ADJ>
-using sense_fn = void (*)(const float*, long long, long long, long long, long long, const float2*, long long,
-                          const float2*, long long, int, int, long long, float2*, float2*, int*);
+using ws_fn = void (*)(const float*, long long, int, int, long long, long long, const float2*, long long, const float2*,
+                       long long, int, int, long long, float2*, float2*, int*);
 template <int ADJ>
-sense_fn<ADJ> sense_kernel_for(int nb) {
+ws_fn<ADJ> ws_kernel_for(int nb) {
   switch (nb) {
-    case 32: return sense_tc_kernel<ADJ, 32>;
-    case 64: return sense_tc_kernel<ADJ, 64>;
-    case 96: return sense_tc_kernel<ADJ, 96>;
-    case 128: return sense_tc_kernel<ADJ, 128>;
-    case 192: return sense_tc_kernel<ADJ, 192>;
-    default: return sense_tc_kernel<ADJ, 256>;
+    case 32: return sense_ws_kernel<ADJ, 32>;
+    case 64: return sense_ws_kernel<ADJ, 64>;
+    case 96: return sense_ws_kernel<ADJ, 96>;
+    case 128: return sense_ws_kernel<ADJ, 128>;
+    default: return sense_ws_kernel<ADJ, 192>;
   }
 }
 
-// kernel attributes (shared memory, carveout) and the forward kernel's resident CTAs per SM
+// kernel attributes (shared memory, carveout) and, for more transmitters than the warp-specialised kernel takes, the
+// forward kernel's resident CTAs per SM
 cisor_status sense_tc_setup(cisor_ctx* c) {
-  const int widths[] = {32, 64, 96, 128, 192, 256};
-  for (int nb : widths) {
-    const int smem = 2 * SPA + 2 * (nb / 8) * SSBO;
-    for (const void* fn : {(const void*)sense_kernel_for<0>(nb), (const void*)sense_kernel_for<1>(nb)}) {
-      CISOR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-      CISOR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    }
+  const int nb = sense_tc_cols(c->T);
+  c->sense_tc_occ = 1;
+  if (sense_tiled(c)) {
+    for (const void* fn : {(const void*)ws_kernel_for<0>(nb), (const void*)ws_kernel_for<1>(nb)})
+      CISOR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ws_smem(nb)));
+    return CISOR_OK;
+  }
+  const int smem = 2 * SPA + 2 * (nb / 8) * SSBO;
+  for (const void* fn : {(const void*)sense_tc_kernel<0, 256>, (const void*)sense_tc_kernel<1, 256>}) {
+    CISOR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CISOR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   }
   int occ = 0;
-  CISOR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sense_kernel_for<0>(sense_tc_cols(c->T)), STH,
-                                                           sense_tc_smem(c->T)));
+  CISOR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sense_tc_kernel<0, 256>, STH, smem));
   c->sense_tc_occ = occ < 1 ? 1 : occ;
   return CISOR_OK;
 }
-
 // splits of the forward GEMM's K (2 Nf floats): at least one wave of resident CTAs, at most S_KMAX floats each;
 // *KS = floats per split (a multiple of SK)
 int sense_tc_splits(const cisor_ctx* c, long long* KS) {
@@ -281,16 +657,67 @@ int sense_tc_splits(const cisor_ctx* c, long long* KS) {
   int S = c->sense_tc_occ * c->sms / mt;
   if (S < 1) S = 1;
   long long ks = ((K + S - 1) / S + SK - 1) / SK * SK;
+  // below four chunks the reduction over more partials costs more than the CTAs save: 32 transmitters, 128 receivers,
+  // 64^2 17.7 us with two, 15.4 with four, 16.9 with eight; 48, 130, 46^2 17.4, 16.9, 18.8
+  if (sense_tiled(c) && ks < 4 * SK) ks = 4 * SK;
   if (ks > S_KMAX) ks = S_KMAX;
   if ((K + ks - 1) / ks > S_MAX) ks = ((K + S_MAX - 1) / S_MAX + SK - 1) / SK * SK;  // bounds the partials
   if (KS) *KS = ks;
   return (int)((K + ks - 1) / ks);
 }
 
+// H, written row-major into sense_h_target(c) by the table kernels, into its final place and form, and Ht from it
+float2* sense_h_target(cisor_ctx* c) { return sense_tiled(c) ? c->Ht : c->H; }
 cisor_status sense_tc_prepare(cisor_ctx* c) {
   if (!c->Ht) return CISOR_OK;
-  const dim3 g((unsigned)((c->Nf + 31) / 32), (unsigned)((c->M + 31) / 32));
-  sense_transpose_kernel<<<g, 256, 0, c->stream>>>(c->H, c->M, c->Nf, c->Ht);
+  const long long Kh = tile_kp(2 * c->Nf);
+  if (sense_tiled(c)) {
+    sense_tile_kernel<<<dim3((unsigned)((Kh / 4 + 255) / 256), (unsigned)(c->M < 4096 ? c->M : 4096)), 256, 0, c->stream>>>(
+        reinterpret_cast<const float*>(c->Ht), c->M, 2 * c->Nf, reinterpret_cast<float*>(c->H));
+    CISOR_CUDA(cudaGetLastError());
+    const dim3 g((unsigned)((c->Nf + 31) / 32), (unsigned)((tile_kp(2 * (long long)c->M) / 2 + 31) / 32));
+    sense_tile_transpose_kernel<<<g, 256, 0, c->stream>>>(reinterpret_cast<const float*>(c->H), c->M, c->Nf,
+                                                          reinterpret_cast<float*>(c->Ht));
+  } else {
+    const dim3 g((unsigned)((c->Nf + 31) / 32), (unsigned)((c->M + 31) / 32));
+    sense_transpose_kernel<<<g, 256, 0, c->stream>>>(c->H, c->M, c->Nf, c->Ht);
+  }
+  CISOR_CUDA(cudaGetLastError());
+  return CISOR_OK;
+}
+
+// rows row0 .. of H, row-major, to device memory
+cisor_status sense_h_rows(cisor_ctx* c, long long row0, long long nrows, float2* out) {
+  if (!sense_tiled(c)) {
+    CISOR_CUDA(cudaMemcpyAsync(out, c->H + row0 * c->Nf, sizeof(float2) * (size_t)nrows * c->Nf,
+                               cudaMemcpyDeviceToDevice, c->stream));
+    return CISOR_OK;
+  }
+  sense_untile_kernel<<<dim3((unsigned)((c->Nf + 255) / 256), (unsigned)(nrows < 4096 ? nrows : 4096)), 256, 0, c->stream>>>(
+      reinterpret_cast<const float*>(c->H), c->M, 2 * c->Nf, row0, nrows, out);
+  CISOR_CUDA(cudaGetLastError());
+  c->launches += 1;
+  return CISOR_OK;
+}
+
+// the GEMM over `rows` rows of the big operand (the context's widest kernel, or the one for fewer transmitters)
+template <int ADJ>
+static cisor_status sense_tc_gemm(cisor_ctx* c, long long rows, long long K, long long KS, int splits,
+                                  const float2* src, long long lds, const float2* f, int ntx, float2* out0,
+                                  float2* out1) {
+  const int rtiles = (int)((rows + 127) / 128);
+  c->tc_used = true;
+  const float* A = reinterpret_cast<const float*>(ADJ ? c->Ht : c->H);
+  if (sense_tiled(c)) {
+    const int nb = sense_tc_cols(c->T), nitems = rtiles * splits;  // (the attributes were set for T's width)
+    ws_kernel_for<ADJ>(nb)<<<nitems < c->sms ? nitems : c->sms, ws_threads(nb), ws_smem(nb), c->stream>>>(
+        A, rows, rtiles, nitems, K, KS, src, lds, f, c->N, ntx, c->M, c->Nf,
+        out0, out1, c->tc_err);
+  } else {
+    sense_tc_kernel<ADJ, 256><<<dim3((unsigned)rtiles, (unsigned)splits), STH, 2 * SPA + 2 * 32 * SSBO, c->stream>>>(
+        A, K, rows, K, KS, src, lds, f, c->N, ntx, c->M, c->Nf, out0,
+        out1, c->tc_err);
+  }
   CISOR_CUDA(cudaGetLastError());
   return CISOR_OK;
 }
@@ -298,26 +725,13 @@ cisor_status sense_tc_prepare(cisor_ctx* c) {
 // partials of Y = H (f .* u) for ntx transmitters into c->sense_part; *splits receives their count
 cisor_status sense_tc_forward(cisor_ctx* c, const float2* f, const float2* u, int ntx, int* splits) {
   long long KS = 0;
-  const int S = sense_tc_splits(c, &KS);
-  const dim3 g((unsigned)((c->M + 127) / 128), (unsigned)S);
-  sense_kernel_for<0>(sense_tc_cols(ntx))<<<g, STH, sense_tc_smem(ntx), c->stream>>>(
-      reinterpret_cast<const float*>(c->H), 2 * c->Nf, c->M, 2 * c->Nf, KS, u, c->Nf, f, c->N, ntx, c->M, c->Nf,
-      c->sense_part, nullptr, c->tc_err);
-  CISOR_CUDA(cudaGetLastError());
-  c->tc_used = true;
-  *splits = S;
-  return CISOR_OK;
+  *splits = sense_tc_splits(c, &KS);
+  return sense_tc_gemm<0>(c, c->M, 2 * c->Nf, KS, *splits, u, c->Nf, f, ntx, c->sense_part, nullptr);
 }
 
 // z = H^H w and b = conj(f) .* z (b may be null) for ntx transmitters
 cisor_status sense_tc_adjoint(cisor_ctx* c, const float2* f, const float2* w, float2* z, float2* b, int ntx) {
-  const dim3 g((unsigned)((c->Nf + 127) / 128));
-  sense_kernel_for<1>(sense_tc_cols(ntx))<<<g, STH, sense_tc_smem(ntx), c->stream>>>(
-      reinterpret_cast<const float*>(c->Ht), 2 * (long long)c->M, c->Nf, 2 * (long long)c->M, 2 * (long long)c->M, w,
-      c->M, f, c->N, ntx, c->M, c->Nf, z, b, c->tc_err);
-  CISOR_CUDA(cudaGetLastError());
-  c->tc_used = true;
-  return CISOR_OK;
+  return sense_tc_gemm<1>(c, c->Nf, 2 * (long long)c->M, 2 * (long long)c->M, 1, w, c->M, f, ntx, z, b);
 }
 
 // after a call that ran the kernels above: an error if one of their waits on the tensor cores gave up.  The

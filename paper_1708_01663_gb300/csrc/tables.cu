@@ -336,9 +336,9 @@ cisor_status build_tables(cisor_ctx* c) {
   if (c->ncomp == 3) {  // vectorial model: dyadic sensing row and polarised plane waves
     CISOR_TRY(vec_tables(c, d_ang, d_rx));
   } else if (d == 3)
-    sensing3d_kernel<<<(unsigned)((MN + 255) / 256), 256, 0, c->stream>>>(c->H, d_rx, c->M, n, c->delta, c->k, c->kb);
+    sensing3d_kernel<<<(unsigned)((MN + 255) / 256), 256, 0, c->stream>>>(sense_h_target(c), d_rx, c->M, n, c->delta, c->k, c->kb);
   else
-    sensing_kernel<<<(unsigned)((MN + 255) / 256), 256, 0, c->stream>>>(c->H, d_rx, c->M, n, c->delta, c->k, c->kb);
+    sensing_kernel<<<(unsigned)((MN + 255) / 256), 256, 0, c->stream>>>(sense_h_target(c), d_rx, c->M, n, c->delta, c->k, c->kb);
   CISOR_CUDA(cudaGetLastError());
   CISOR_TRY(sense_tc_prepare(c));
   const unsigned gT = (unsigned)((TN + 255) / 256);

@@ -312,7 +312,7 @@ __global__ void polarised_wave_kernel(float2* u, const double* tx, int T, int n,
 
 cisor_status vec_tables(cisor_ctx* c, const double* d_tx, const double* d_rx) {
   const long long MK = (long long)c->M * c->Nf, TK = (long long)c->T * c->Nf;
-  dyadic_sensing_kernel<<<(unsigned)((MK + 255) / 256), 256, 0, c->stream>>>(c->H, d_rx, c->M, c->n, c->delta, c->k);
+  dyadic_sensing_kernel<<<(unsigned)((MK + 255) / 256), 256, 0, c->stream>>>(sense_h_target(c), d_rx, c->M, c->n, c->delta, c->k);
   CISOR_CUDA(cudaGetLastError());
   polarised_wave_kernel<<<(unsigned)((TK + 255) / 256), 256, 0, c->stream>>>(c->u_in, d_tx, c->T, c->n, c->delta, c->k);
   CISOR_CUDA(cudaGetLastError());
