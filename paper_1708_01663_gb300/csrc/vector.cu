@@ -28,34 +28,8 @@
 
 namespace cisor {
 
-// (D F)^(C) at voxel v = (ix, iy, iz) of the 3-component field F (component stride N)
-template <int C>
-__device__ __forceinline__ float2 graddiv_at(const float2* __restrict__ F, int N, int n, int ix, int iy, int iz, int v,
-                                            float inv_d2) {
-  const int coord[3] = {ix, iy, iz};
-  const int stride[3] = {1, n, n * n};
-  const float2* Fc = F + C * N;
-  float2 acc = c_scale(Fc[v], -2.f);
-  if (coord[C] > 0) acc = c_add(acc, Fc[v - stride[C]]);
-  if (coord[C] < n - 1) acc = c_add(acc, Fc[v + stride[C]]);
-  acc = c_scale(acc, inv_d2);
-  float2 mix = make_float2(0.f, 0.f);
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    if (j == C) continue;
-    const float2* Fj = F + j * N;
-#pragma unroll
-    for (int sc = -1; sc <= 1; sc += 2)
-#pragma unroll
-      for (int sj = -1; sj <= 1; sj += 2) {
-        const int qc = coord[C] + sc, qj = coord[j] + sj;
-        if (qc < 0 || qc >= n || qj < 0 || qj >= n) continue;
-        const float2 val = Fj[v + sc * stride[C] + sj * stride[j]];
-        mix = (sc * sj > 0) ? c_add(mix, val) : c_sub(mix, val);
-      }
-  }
-  return c_add(acc, c_scale(mix, 0.25f * inv_d2));
-}
+// what a stencil pass does with (D F): the adjoint's pre-pass, or A x (b - A x) without and with inner products
+enum { VEC_PRE = -1 };
 
 struct VecEpiArgs {
   const float2* C;      // conv output [ntx, 3, N] (forward) or the field x (pre-pass)
@@ -63,61 +37,114 @@ struct VecEpiArgs {
   const float2* aux;
   float2* out;
   float2* out2;
-  int epi;              // EPI_MATVEC, EPI_RESID; -1: pre-pass w = x + D x / k^2
+  int epi;              // EPI_MATVEC, EPI_RESID; VEC_PRE: pre-pass w = x + D x / k^2
+  int need_aux;
   int dot_a[DOT_SLOTS], dot_b[DOT_SLOTS];
   const int* active;
   float* part;
-  int n, RB, nblk;
+  int n, nblk;
   long long N;
   float inv_k2, inv_d2;
 };
 
-// RB x rows (RB n voxels) of component C of transmitter blockIdx.z (N < 2^31: n <= 64).
-template <int C>
-__device__ __forceinline__ void vec_stencil_body(const VecEpiArgs& a) {
-  const int rb = blockIdx.x, t = blockIdx.z;
-  const int N = (int)a.N, n = a.n;
+constexpr int VS_Z = 4;  // output planes per CTA (of 4, 8, 16: 8 is 1% faster at 32^3, 4 by 8% at 16^3)
+
+// All three components of 256 (x, y) columns over VS_Z planes of transmitter blockIdx.z; a thread marches along z.
+// The mixed derivatives along z are differences over z of in-plane differences,
+//     (D F)^(x) ~ M0(z + 1) - M0(z - 1),  M0 = F2(x + 1) - F2(x - 1)   (1 / 4 delta^2; y likewise, z from F0 and F1),
+// so a plane's values are read once and kept as M0, M1, M2 and the centre of F2 for the three planes they act on: 19
+// reads a voxel for the three components instead of 33, one set of bounds tests, and no component's field read by
+// three CTAs (one component a CTA took 15 plane reads through L2 for the 3 it needs).  Bound by memory: C, x and the
+// result are 64 MB each at 81 transmitters, 32^3, 28 us at the copy rate.  There a pass fell from 65 us to 36 (A x) and
+// 41 (pre-pass), A x as a whole from 315 to 287, A^H x from 302 to 279; with 16 transmitters 68 to 64 and 66 to 60.
+// Three CTAs an SM (80 registers): two hide less (293 / 289), four spill (310 / 301).
+template <int DK>
+__global__ void __launch_bounds__(256, 3) vec_stencil_kernel(const VecEpiArgs a) {
+  const int t = blockIdx.z;
+  if (a.active && !a.active[t]) return;
+  const int N = (int)a.N, n = a.n, n2 = n * n;
+  const int col = blockIdx.x * 256 + threadIdx.x, z0 = blockIdx.y * VS_Z, z1 = min(n, z0 + VS_Z);
   const long long base = (long long)t * 3 * N;
-  const float2* F = a.C + base;
-  const int v0 = rb * a.RB * n;
-  const int v1 = min(N, v0 + a.RB * n);
-  const bool any_dot = a.epi >= 0 && (a.dot_a[0] | a.dot_a[1] | a.dot_a[2]) != 0;
-  const bool need_aux = a.epi == EPI_RESID || a.dot_a[0] == OP_AUX || a.dot_b[0] == OP_AUX ||
-                        a.dot_a[1] == OP_AUX || a.dot_b[1] == OP_AUX || a.dot_a[2] == OP_AUX || a.dot_b[2] == OP_AUX;
   float2 acc[DOT_SLOTS];
 #pragma unroll
   for (int s = 0; s < DOT_SLOTS; ++s) acc[s] = make_float2(0.f, 0.f);
-  for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
-    const int row = v / n, ix = v - row * n, iz = row / n, iy = row - iz * n;
-    const float2 dc = graddiv_at<C>(F, N, n, ix, iy, iz, v, a.inv_d2);
-    const long long idx = base + (long long)C * N + v;
-    if (a.epi < 0) {  // pre-pass of the adjoint: w = x + D x / k^2
-      a.out[idx] = c_add(F[C * N + v], c_scale(dc, a.inv_k2));
-      continue;
-    }
-    const float2 xv = a.x[idx];
-    float2 y = c_sub(c_sub(xv, F[C * N + v]), c_scale(dc, a.inv_k2));
-    const float2 av = need_aux ? a.aux[idx] : make_float2(0.f, 0.f);
-    if (a.epi == EPI_RESID) y = c_sub(av, y);
-    a.out[idx] = y;
-    if (a.out2) a.out2[idx] = y;
-    if (any_dot) {
+  if (col < n2) {
+    const int iy = col / n, ix = col - iy * n;
+    const bool xl = ix > 0, xr = ix < n - 1, yl = iy > 0, yr = iy < n - 1;
+    const float2* F0 = a.C + base + (long long)z0 * n2 + col;  // plane z0; planes z0 - 1 .. z1 by offset
+    const float2 *F1 = F0 + N, *F2 = F1 + N;
+    const float2 zero = make_float2(0.f, 0.f);
+    auto at = [&](const float2* p, int o, bool in) { return in ? __ldg(p + o) : zero; };
+    const float q = 0.25f * a.inv_d2;
+    // of the plane before, this one and the next
+    float2 m0[3], m1[3], m2[3], c2[3], c0, c1, d0, d1;
+    auto load = [&](int z, float2& M0, float2& M1, float2& M2, float2& C2, float2& C0, float2& C1, float2& D0, float2& D1) {
+      const bool in = z >= 0 && z < n;
+      const int o = (z - z0) * n2;
+      const bool l = in && xl, r = in && xr, b = in && yl, u = in && yr;
+      const float2 e0 = at(F0, o - 1, l), e1 = at(F0, o + 1, r), g0 = at(F1, o - n, b), g1 = at(F1, o + n, u);
+      C0 = at(F0, o, in);
+      C1 = at(F1, o, in);
+      C2 = at(F2, o, in);
+      M0 = c_sub(at(F2, o + 1, r), at(F2, o - 1, l));
+      M1 = c_sub(at(F2, o + n, u), at(F2, o - n, b));
+      M2 = c_add(c_sub(e1, e0), c_sub(g1, g0));
+      if (z >= z0 && z < z1) {  // the in-plane parts of components x and y
+        D0 = c_add(c_scale(c_add(c_scale(C0, -2.f), c_add(e0, e1)), a.inv_d2),
+                   c_scale(c_sub(c_sub(at(F1, o + 1 + n, r && u), at(F1, o + 1 - n, r && b)),
+                                 c_sub(at(F1, o - 1 + n, l && u), at(F1, o - 1 - n, l && b))), q));
+        D1 = c_add(c_scale(c_add(c_scale(C1, -2.f), c_add(g0, g1)), a.inv_d2),
+                   c_scale(c_sub(c_sub(at(F0, o + 1 + n, r && u), at(F0, o + 1 - n, r && b)),
+                                 c_sub(at(F0, o - 1 + n, l && u), at(F0, o - 1 - n, l && b))), q));
+      }
+    };
+    float2 n0, n1, nd0, nd1;
+    load(z0 - 1, m0[0], m1[0], m2[0], c2[0], n0, n1, nd0, nd1);
+    load(z0, m0[1], m1[1], m2[1], c2[1], c0, c1, d0, d1);
+#pragma unroll 2
+    for (int z = z0; z < z1; ++z) {
+      const long long i0 = base + (long long)z * n2 + col;
+      float2 xv[3], av[3];  // (read before the stores, which the compiler must take for aliases)
+      if (DK != VEC_PRE) {
 #pragma unroll
-      for (int s = 0; s < DOT_SLOTS; ++s)
-        if (a.dot_a[s]) acc[s] = c_add(acc[s], c_cjmul(pick(a.dot_a[s], y, xv, av), pick(a.dot_b[s], y, xv, av)));
+        for (int c = 0; c < 3; ++c) {
+          xv[c] = a.x[i0 + (long long)c * N];
+          av[c] = a.need_aux ? a.aux[i0 + (long long)c * N] : zero;
+        }
+      }
+      load(z + 1, m0[2], m1[2], m2[2], c2[2], n0, n1, nd0, nd1);
+      const float2 dc[3] = {c_add(d0, c_scale(c_sub(m0[2], m0[0]), q)), c_add(d1, c_scale(c_sub(m1[2], m1[0]), q)),
+                            c_add(c_scale(c_add(c_scale(c2[1], -2.f), c_add(c2[0], c2[2])), a.inv_d2),
+                                  c_scale(c_sub(m2[2], m2[0]), q))};
+      const float2 ctr[3] = {c0, c1, c2[1]};
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const long long idx = i0 + (long long)c * N;
+        if (DK == VEC_PRE) {  // pre-pass of the adjoint: w = x + D x / k^2
+          a.out[idx] = c_add(ctr[c], c_scale(dc[c], a.inv_k2));
+        } else {
+          float2 y = c_sub(c_sub(xv[c], ctr[c]), c_scale(dc[c], a.inv_k2));
+          if (a.epi == EPI_RESID) y = c_sub(av[c], y);
+          a.out[idx] = y;
+          if (a.out2) a.out2[idx] = y;
+          if (DK == DOTS_ANY) {
+#pragma unroll
+            for (int s = 0; s < DOT_SLOTS; ++s)
+              if (a.dot_a[s]) acc[s] = c_add(acc[s], c_cjmul(pick(a.dot_a[s], y, xv[c], av[c]), pick(a.dot_b[s], y, xv[c], av[c])));
+          }
+        }
+      }
+      m0[0] = m0[1], m1[0] = m1[1], m2[0] = m2[1], c2[0] = c2[1];
+      m0[1] = m0[2], m1[1] = m1[2], m2[1] = m2[2], c2[1] = c2[2];
+      c0 = n0, c1 = n1, d0 = nd0, d1 = nd1;
     }
   }
-  if (any_dot)
-    block_dots<256>(acc, reinterpret_cast<float2*>(a.part) + (((size_t)t * 3 + C) * a.nblk + rb) * DOT_SLOTS);
-}
-
-// One CTA: RB x rows of component blockIdx.y of transmitter blockIdx.z.
-__global__ void __launch_bounds__(256) vec_stencil_kernel(const VecEpiArgs a) {
-  if (a.active && !a.active[blockIdx.z]) return;
-  switch (blockIdx.y) {
-    case 0: vec_stencil_body<0>(a); break;
-    case 1: vec_stencil_body<1>(a); break;
-    default: vec_stencil_body<2>(a); break;
+  if (DK == DOTS_ANY) {  // a partial per CTA, zeros in the other slots of the transmitter's 3 nblk
+    float2* part = reinterpret_cast<float2*>(a.part) + (size_t)t * 3 * a.nblk * DOT_SLOTS;
+    const int cta = blockIdx.y * gridDim.x + blockIdx.x, ctas = gridDim.x * gridDim.y;
+    block_dots<256>(acc, part + (size_t)cta * DOT_SLOTS);
+    for (int b = cta + ctas; b < 3 * a.nblk; b += ctas)
+      if (threadIdx.x < DOT_SLOTS) part[(size_t)b * DOT_SLOTS + threadIdx.x] = make_float2(0.f, 0.f);
   }
 }
 
@@ -125,7 +152,6 @@ static VecEpiArgs stencil_args(cisor_ctx* c) {
   VecEpiArgs a{};
   a.n = c->n;
   a.N = c->N;
-  a.RB = conv_rows_per_block(c->dim, c->P);
   a.nblk = c->nblk;
   a.part = c->part;
   a.inv_k2 = (float)(1.0 / (c->k * c->k));
@@ -134,8 +160,14 @@ static VecEpiArgs stencil_args(cisor_ctx* c) {
 }
 
 static cisor_status launch_stencil(cisor_ctx* c, const VecEpiArgs& a, int ntx) {
-  dim3 g(c->nblk, 3, ntx);
-  vec_stencil_kernel<<<g, 256, 0, c->stream>>>(a);
+  // (at most 3 nblk CTAs a transmitter, the slots of its partials: nblk is n^2 / 32 or more)
+  const dim3 g((unsigned)((c->n * c->n + 255) / 256), (unsigned)((c->n + VS_Z - 1) / VS_Z), ntx);
+  if (a.epi == VEC_PRE)
+    vec_stencil_kernel<VEC_PRE><<<g, 256, 0, c->stream>>>(a);
+  else if (a.dot_a[0] | a.dot_a[1] | a.dot_a[2])
+    vec_stencil_kernel<DOTS_ANY><<<g, 256, 0, c->stream>>>(a);
+  else
+    vec_stencil_kernel<DOTS_NONE><<<g, 256, 0, c->stream>>>(a);
   CISOR_CUDA(cudaGetLastError());
   c->launches += 1;
   return CISOR_OK;
@@ -165,13 +197,15 @@ cisor_status vec_matvec(cisor_ctx* c, const VecOp& op) {
       a.dot_a[s] = op.dot_a[s];
       a.dot_b[s] = op.dot_b[s];
     }
+    a.need_aux = op.epilogue == EPI_RESID;
+    for (int s = 0; s < DOT_SLOTS; ++s) a.need_aux |= op.dot_a[s] == OP_AUX || op.dot_b[s] == OP_AUX;
     a.active = op.active;
     return launch_stencil(c, a, op.ntx);
   }
   VecEpiArgs a = stencil_args(c);
   a.C = op.x;
   a.out = c->vbuf;
-  a.epi = -1;
+  a.epi = VEC_PRE;
   a.active = op.active;
   CISOR_TRY(launch_stencil(c, a, op.ntx));
   ConvOp co{};
@@ -202,7 +236,7 @@ cisor_status vec_gz(cisor_ctx* c) {
   VecEpiArgs a = stencil_args(c);
   a.C = c->vadj;
   a.out = c->vbuf;
-  a.epi = -1;
+  a.epi = VEC_PRE;
   CISOR_TRY(launch_stencil(c, a, c->T));
   ConvOp co{};
   co.adjoint = 1;
