@@ -28,7 +28,7 @@
 
 namespace cisor {
 
-// what a stencil pass does with (D F): the adjoint's pre-pass, or A x (b - A x) without and with inner products
+// besides the inner products (DOTS_NONE .. DOTS_ANY) of an A x pass: the adjoint's pre-pass
 enum { VEC_PRE = -1 };
 
 struct VecEpiArgs {
@@ -58,6 +58,8 @@ constexpr int VS_Z = 4;  // output planes per CTA (of 4, 8, 16: 8 is 1% faster a
 // result are 64 MB each at 81 transmitters, 32^3, 28 us at the copy rate.  There a pass fell from 65 us to 36 (A x) and
 // 41 (pre-pass), A x as a whole from 315 to 287, A^H x from 302 to 279; with 16 transmitters 68 to 64 and 66 to 60.
 // Three CTAs an SM (80 registers): two hide less (293 / 289), four spill (310 / 301).
+// The solver's sets of inner products are compiled in (dots.cuh; a pass with them 53 us by operand codes, the gradient
+// of 81 transmitters 8.09 -> 7.96 ms).
 template <int DK>
 __global__ void __launch_bounds__(256, 3) vec_stencil_kernel(const VecEpiArgs a) {
   const int t = blockIdx.z;
@@ -101,7 +103,8 @@ __global__ void __launch_bounds__(256, 3) vec_stencil_kernel(const VecEpiArgs a)
     float2 n0, n1, nd0, nd1;
     load(z0 - 1, m0[0], m1[0], m2[0], c2[0], n0, n1, nd0, nd1);
     load(z0, m0[1], m1[1], m2[1], c2[1], c0, c1, d0, d1);
-#pragma unroll 2
+constexpr int UN = DK > DOTS_NONE ? 1 : 2;  // (inner products leave no registers for two planes)
+#pragma unroll UN
     for (int z = z0; z < z1; ++z) {
       const long long i0 = base + (long long)z * n2 + col;
       float2 xv[3], av[3];  // (read before the stores, which the compiler must take for aliases)
@@ -109,7 +112,7 @@ __global__ void __launch_bounds__(256, 3) vec_stencil_kernel(const VecEpiArgs a)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           xv[c] = a.x[i0 + (long long)c * N];
-          av[c] = a.need_aux ? a.aux[i0 + (long long)c * N] : zero;
+          av[c] = DK == DOTS_RV || DK == DOTS_RES || a.need_aux ? a.aux[i0 + (long long)c * N] : zero;
         }
       }
       load(z + 1, m0[2], m1[2], m2[2], c2[2], n0, n1, nd0, nd1);
@@ -127,7 +130,9 @@ __global__ void __launch_bounds__(256, 3) vec_stencil_kernel(const VecEpiArgs a)
           if (a.epi == EPI_RESID) y = c_sub(av[c], y);
           a.out[idx] = y;
           if (a.out2) a.out2[idx] = y;
-          if (DK == DOTS_ANY) {
+          if constexpr (DK > DOTS_NONE && DK < DOTS_ANY) {
+            dots_accumulate<DK>(ConvOp{}, acc, y, xv[c], av[c]);  // (fixed operands: the codes are not read)
+          } else if constexpr (DK == DOTS_ANY) {
 #pragma unroll
             for (int s = 0; s < DOT_SLOTS; ++s)
               if (a.dot_a[s]) acc[s] = c_add(acc[s], c_cjmul(pick(a.dot_a[s], y, xv[c], av[c]), pick(a.dot_b[s], y, xv[c], av[c])));
@@ -139,10 +144,10 @@ __global__ void __launch_bounds__(256, 3) vec_stencil_kernel(const VecEpiArgs a)
       c0 = n0, c1 = n1, d0 = nd0, d1 = nd1;
     }
   }
-  if (DK == DOTS_ANY) {  // a partial per CTA, zeros in the other slots of the transmitter's 3 nblk
+  if constexpr (DK > DOTS_NONE) {  // a partial per CTA, zeros in the other slots of the transmitter's 3 nblk
     float2* part = reinterpret_cast<float2*>(a.part) + (size_t)t * 3 * a.nblk * DOT_SLOTS;
     const int cta = blockIdx.y * gridDim.x + blockIdx.x, ctas = gridDim.x * gridDim.y;
-    block_dots<256>(acc, part + (size_t)cta * DOT_SLOTS);
+    block_dots<256, DotSlots<DK>::MASK>(acc, part + (size_t)cta * DOT_SLOTS);
     for (int b = cta + ctas; b < 3 * a.nblk; b += ctas)
       if (threadIdx.x < DOT_SLOTS) part[(size_t)b * DOT_SLOTS + threadIdx.x] = make_float2(0.f, 0.f);
   }
@@ -162,12 +167,19 @@ static VecEpiArgs stencil_args(cisor_ctx* c) {
 static cisor_status launch_stencil(cisor_ctx* c, const VecEpiArgs& a, int ntx) {
   // (at most 3 nblk CTAs a transmitter, the slots of its partials: nblk is n^2 / 32 or more)
   const dim3 g((unsigned)((c->n * c->n + 255) / 256), (unsigned)((c->n + VS_Z - 1) / VS_Z), ntx);
-  if (a.epi == VEC_PRE)
-    vec_stencil_kernel<VEC_PRE><<<g, 256, 0, c->stream>>>(a);
-  else if (a.dot_a[0] | a.dot_a[1] | a.dot_a[2])
-    vec_stencil_kernel<DOTS_ANY><<<g, 256, 0, c->stream>>>(a);
-  else
-    vec_stencil_kernel<DOTS_NONE><<<g, 256, 0, c->stream>>>(a);
+  ConvOp dots{};
+  for (int k = 0; k < DOT_SLOTS; ++k) {
+    dots.dot_a[k] = a.dot_a[k];
+    dots.dot_b[k] = a.dot_b[k];
+  }
+  switch (a.epi == VEC_PRE ? (int)VEC_PRE : dots_kind(dots)) {
+    case VEC_PRE: vec_stencil_kernel<VEC_PRE><<<g, 256, 0, c->stream>>>(a); break;
+    case DOTS_NONE: vec_stencil_kernel<DOTS_NONE><<<g, 256, 0, c->stream>>>(a); break;
+    case DOTS_RV: vec_stencil_kernel<DOTS_RV><<<g, 256, 0, c->stream>>>(a); break;
+    case DOTS_TS: vec_stencil_kernel<DOTS_TS><<<g, 256, 0, c->stream>>>(a); break;
+    case DOTS_RES: vec_stencil_kernel<DOTS_RES><<<g, 256, 0, c->stream>>>(a); break;
+    default: vec_stencil_kernel<DOTS_ANY><<<g, 256, 0, c->stream>>>(a);
+  }
   CISOR_CUDA(cudaGetLastError());
   c->launches += 1;
   return CISOR_OK;
