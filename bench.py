@@ -355,9 +355,10 @@ def run_reference(args):
 
 
 def conv_sources_hash():
-    """Hash of the sources of the convolution kernels (conv.cu, conv_cluster.cu, regfft.cuh, fft.cuh, dots.cuh)."""
+    """Hash of the sources of the convolution kernels (conv.cu, conv_cluster.cu, conv3d.cu, plane_layout.cuh,
+    regfft.cuh, fft.cuh, dots.cuh)."""
     h = hashlib.sha256()
-    for name in ("conv.cu", "conv_cluster.cu", "regfft.cuh", "fft.cuh", "dots.cuh"):
+    for name in ("conv.cu", "conv_cluster.cu", "conv3d.cu", "plane_layout.cuh", "regfft.cuh", "fft.cuh", "dots.cuh"):
         with open(os.path.join(ROOT, "paper_1708_01663_gb300", "csrc", name), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -789,8 +790,8 @@ def main():
             "roofline": {"bound": "alu", "achieved": achieved_tf, "peak": fp32_peak, "unit": "TFLOP/s",
                          "frac": achieved_tf / fp32_peak, "traffic": traffic,
                          "kernel": "batched FFT matvec A x over all T (conv_rows_fwd + conv_cols + conv_rows_inv)"
-                                   if dim == 2 else "batched FFT matvec A x over all T (conv_rows_fwd + conv_cols "
-                                   "y-forward + conv_cols z-spectrum + conv_cols y-inverse + conv_rows_inv"
+                                   if dim == 2 else "batched FFT matvec A x over all T (conv3_rows_fwd + conv3_plane "
+                                   "+ conv3_rows_inv"
                                    + (" per field component, + the grad-div stencil)" if vec else ")"),
                          "ms_per_launch": mv_ms, "alg_flops_per_launch": alg_flops,
                          "alg_bytes_per_launch": alg_bytes,

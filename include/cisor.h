@@ -268,7 +268,9 @@ cisor_status cisor_apply_A_static(const void* ghat_scaled, const void* f, const 
  * two-stage kernel (shape code 16: one shared-memory exchange per transform;
  * 512 = 32 x 16 on 2D grids, 256 = 16 x 16 and 128 = 16 x 8 on 2D and 3D
  * grids; none at P = 64), on this context's sizes, `reps` batched matvecs
- * each with CUDA events, and keeps the fastest.  *cols_nt_out (may be NULL)
+ * each with CUDA events, and keeps the fastest.  3D grids with P <= 128 have no
+ * separate column kernels (one kernel transforms whole planes): there the
+ * shape changes nothing.  *cols_nt_out (may be NULL)
  * receives the chosen shape code (512, 256 or 16).  Results agree to FP32
  * rounding whichever shape runs. */
 cisor_status cisor_autotune(cisor_ctx* ctx, int reps, int* cols_nt_out);

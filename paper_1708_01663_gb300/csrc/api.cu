@@ -1,8 +1,11 @@
-// C ABI entry points (include/cisor.h).  Arguments are copied into the
-// context's device buffers with cudaMemcpyDefault (unified addressing: host
-// or device pointers), work runs on the context's own non-blocking stream,
-// ordered after and before the caller's stream with events, and results are
-// copied out; a call that writes host memory synchronises before returning.
+// C ABI entry points (include/cisor.h).  The operators (cisor_apply_A,
+// cisor_sense, cisor_sense_adjoint, cisor_tv_prox) read and write device
+// arguments where they are (Call::operand, in_place); host memory, arguments
+// that overlap an output, and what a solve keeps (f, y, the state) are copied
+// to and from the context's device buffers with cudaMemcpyDefault (unified
+// addressing).  Work runs on the context's own non-blocking stream, ordered
+// after and before the caller's stream with events; a call that writes host
+// memory synchronises before returning.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>

@@ -9,7 +9,8 @@
 //  grad_assemble : g = sum_t conj(u_t) .* (z_t + G^H v_t)        (Eq. 12 before Re)
 //                  and the gradient step s - gamma grad D        (Eq. 9 argument)
 // The GEMMs run on the tensor cores (TF32 hi / lo products, sense_tc.cu) where
-// the sizes allow it (T <= 128, even M and field length) and otherwise on the
+// the sizes allow it (T <= 128, even M and field length; up to 96 transmitters
+// with H stored as the tiles they stream) and otherwise on the
 // FP32 pipes with the tiles below; a single TF32 product would break the 1e-5
 // sensing parity.
 #include <math.h>

@@ -17,7 +17,10 @@
 //   rho' , beta, convergence / iteration cap / breakdown         scalar
 // A transmitter whose recursive residual reaches tol is masked off (its CTAs
 // exit at once).  Chunks of iterations are captured once into a CUDA graph
-// and replayed; the host reads one counter per chunk.  At the end the true
+// and replayed; the host reads the transmitters' states from mapped memory
+// after each.  A cold start (x = 0) takes r = b without a pass, and the last
+// residual pass of an adjoint solve also stores the z + G^H v of the
+// gradient.  At the end the true
 // residual ||b - A x|| / ||b|| is recomputed with an explicit matvec and any
 // transmitter above tol restarts from its current iterate (the stopping rule
 // is always on the true residual of the paper's system).

@@ -7,9 +7,10 @@
 //     p_k     = Pi_unit-disk(r_k + D x(r_k) / (8 lam))
 //     t_{k+1} = (1 + sqrt(1 + 4 t_k^2)) / 2
 //     r_{k+1} = p_k + ((t_k - 1) / t_{k+1}) (p_k - p_{k-1})
-// from r_1 = p_0 = 0, t_1 = 1; output x(p_K).  One kernel per FGP iteration
-// (r ping-pongs between two buffers; p is updated in place per pixel); the
-// right neighbour's x comes from the next lane by warp shuffle.  Complex f
+// from r_1 = p_0 = 0, t_1 = 1; output x(p_K).  2D: several iterations per
+// kernel on image tiles with a halo (tv_block_kernel); 3D: one kernel per
+// iteration (r ping-pongs between two buffers; p is updated in place per
+// pixel), the right neighbour's x by warp shuffle.  Complex f
 // takes the separable prox: Re and Im planes, each with its own box.
 // The last kernel also applies the relaxed-FISTA momentum of Eq. 11,
 // s_{k+1} = f_k + beta (f_k - f_{k-1}).

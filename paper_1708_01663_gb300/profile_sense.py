@@ -14,7 +14,7 @@ L2 error of both products against FP64 products of the context's own H on
 the GPU (torch, complex128).  A launch list of the same
 command: ``ncu --clock-control none --metrics gpu__time_duration.sum -k
 regex:sense -c 20``; a full-metric capture names one kernel
-(``-k regex:sense_tc_kernel``) and one or two launches, on a small ``--n``.
+(``-k regex:sense_ws_kernel``) and one or two launches, on a small ``--n``.
 """
 from __future__ import annotations
 
