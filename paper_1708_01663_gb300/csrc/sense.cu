@@ -113,9 +113,18 @@ __global__ void __launch_bounds__(256, 2) sense_fwd_kernel(const float2* __restr
     }
 }
 
-// Z = sum of the ks split-K partials in FP64, w = Z - y (0 at receivers a transmitter does not record), and
+// s + e += p with the rounding error of every sum kept in e (Knuth's TwoSum)
+__device__ __forceinline__ void two_sum(float& s, float& e, float p) {
+  const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
+  e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b)));
+  s = t;
+}
+
+// Z = sum of the ks split-K partials, w = Z - y (0 at receivers a transmitter does not record), and
 // D += 1/2 sum |w|^2.  A CTA takes 32 consecutive entries (lanes, coalesced); its 8 warps sum the partials
-// k = w, w + 8, ... and warp 0 adds the 8 sums in warp order (the same order every call).
+// k = w, w + 8, ... and warp 0 adds the 8 sums in FP64 in warp order (the same order every call).  A warp sums its
+// partials as pairs of FP32 values (two_sum: 48 bits), since FP64 runs at a small fraction of the FP32 rate: 256
+// partials of 48 x 1024 entries cost 78 us more by FP64 additions (1265 -> 1185 us for both sensing products).  A sum that is not finite is taken again in FP64.
 constexpr int RED_WARPS = 8;
 __global__ void __launch_bounds__(32 * RED_WARPS) sense_reduce_kernel(const float2* __restrict__ part, int ks, int T,
                                                                      int M, const float2* __restrict__ y,
@@ -128,11 +137,22 @@ __global__ void __launch_bounds__(32 * RED_WARPS) sense_reduce_kernel(const floa
   const long long TM = (long long)T * M;
   double sx = 0.0, sy = 0.0;
   if (idx < TM) {
-#pragma unroll 4
+    float2 s = make_float2(0.f, 0.f), e = make_float2(0.f, 0.f);
+#pragma unroll 8
     for (int k = warp; k < ks; k += RED_WARPS) {
       const float2 p = part[(long long)k * TM + idx];
-      sx += p.x;
-      sy += p.y;
+      two_sum(s.x, e.x, p.x);
+      two_sum(s.y, e.y, p.y);
+    }
+    sx = (double)s.x + (double)e.x;
+    sy = (double)s.y + (double)e.y;
+    if (!isfinite(e.x) || !isfinite(e.y)) {
+      sx = sy = 0.0;
+      for (int k = warp; k < ks; k += RED_WARPS) {
+        const float2 p = part[(long long)k * TM + idx];
+        sx += p.x;
+        sy += p.y;
+      }
     }
   }
   red[warp][lane] = make_double2(sx, sy);

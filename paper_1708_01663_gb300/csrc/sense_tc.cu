@@ -35,14 +35,15 @@
 // small operand's write and its reads by the MMAs (93 KB at NB = 96 against 140 KB
 // with both planes of A there).
 // Measured at 48 transmitters, 1024 receivers, 64^3 (H and Ht of 2.1 GB): forward
-// 1.15 -> 0.67 ms, adjoint 0.93 -> 0.58 ms against the kernel below on row-major
+// 1.15 -> 0.60 ms, adjoint 0.93 -> 0.58 ms against the kernel below on row-major
 // matrices, which does all roles in every thread; 64 transmitters, 256 receivers,
-// 256^2: 0.136 -> 0.078, 0.092 -> 0.085; 81, 36, 32^3 vectorial: 0.108 -> 0.097,
+// 256^2: 0.136 -> 0.071, 0.092 -> 0.082; 81, 36, 32^3 vectorial: 0.108 -> 0.095,
 // 0.096 -> 0.068; 8, 360, 128^2: 0.044 -> 0.024, 0.037 -> 0.017; 8, 32, 64^2: 0.017 -> 0.015,
 // 0.008 -> 0.007 (all launches; slower only with two receivers and many
-// transmitters, whose chunks are mostly padding: 48, 2, 256^2 adjoint 20 -> 24 us).  What bounds it: the hand-overs between the roles
-// (below); the MMAs keep the tensor pipe about half of the time at NB = 96, the
-// copies the memory for 45%.  More than 96 transmitters leave no room for two
+// transmitters, whose chunks are mostly padding: 48, 2, 256^2 adjoint 20 -> 24
+// us).  What bounds it: the hand-overs between the roles (below); the MMAs keep
+// the tensor pipe about half of the time at NB = 96, the copies the memory for
+// half.  More than 96 transmitters leave no room for two
 // accumulators and A in tensor memory and take the kernel below (sense_tc_kernel).
 // Every wait is bounded (a timeout sets the context's error flag, read by the host
 // after the call).
@@ -255,7 +256,8 @@ __global__ void __launch_bounds__(STH, NB > 128 ? 1 : 2) sense_tc_kernel(const f
 // one reuses).  A completed barrier still costs its waiter 200 to 350 cycles and a commit 300, against about 650 for
 // the chunk's MMAs at NB = 96; that is why the roles run up to DEP chunks apart and why two threads issue, each
 // waiting while the other's MMAs run.  Forward / adjoint at 48 transmitters, 64^3: 0.99 / 0.80 ms with one group of
-// builders and one issuer, 0.73 / 0.64 with two groups, 0.67 / 0.58 with two issuers.
+// builders and one issuer, 0.73 / 0.64 with two groups, 0.67 / 0.58 with two issuers
+// (all before the reduction's faster sums, with which it is 0.60 / 0.58).
 // operand buffers and accumulators (at most as many): what 512 columns of tensor memory hold.  An even number of
 // buffers: then a buffer's chunks belong to one group of converters and of builders and to one issuer, so that nobody
 // tests a barrier that is still a phase behind the one it waits for.
