@@ -262,13 +262,28 @@ __global__ void __launch_bounds__(256, 2) sense_adj_kernel(const float2* __restr
     }
 }
 
-__global__ void __launch_bounds__(256) grad_kernel(const float2* __restrict__ u, const float2* __restrict__ gz, int T,
-                                                   long long N, const float2* __restrict__ s, float gamma, int complex_f,
-                                                   float2* __restrict__ grad, float2* __restrict__ zstep) {
-  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
+// A CTA takes 32 consecutive entries (lanes), its warps the transmitters t = w, w + 8, ...; warp 0 adds the 8 sums in
+// warp order.  Bound by memory, 16 bytes per entry and transmitter: with a thread per entry for all transmitters a
+// small grid left most of the chip idle (81 x 3 fields of 32^3: 95 us at 128 CTAs against
+// 19 at the copy rate; the vectorial gradient now takes 75 us less, 64 fields of 256^2 12 us less, 8 of 128^2 the same).
+constexpr int GRAD_WARPS = 8;
+__global__ void __launch_bounds__(32 * GRAD_WARPS) grad_kernel(const float2* __restrict__ u, const float2* __restrict__ gz,
+                                                              int T, long long N, const float2* __restrict__ s, float gamma,
+                                                              int complex_f, float2* __restrict__ grad,
+                                                              float2* __restrict__ zstep) {
+  __shared__ float2 part[GRAD_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long n = (long long)blockIdx.x * 32 + lane;
   float2 g = make_float2(0.f, 0.f);
-  for (int t = 0; t < T; ++t) g = c_add(g, c_cjmul(u[(long long)t * N + n], gz[(long long)t * N + n]));
+  if (n < N) {
+#pragma unroll 4
+    for (int t = warp; t < T; t += GRAD_WARPS) g = c_add(g, c_cjmul(u[(long long)t * N + n], gz[(long long)t * N + n]));
+  }
+  part[warp][lane] = g;
+  __syncthreads();
+  if (warp != 0 || n >= N) return;
+#pragma unroll
+  for (int w = 1; w < GRAD_WARPS; ++w) g = c_add(g, part[w][lane]);
   if (grad) grad[n] = g;
   if (zstep) {
     const float2 sv = s[n];
@@ -345,7 +360,7 @@ cisor_status sense_adjoint(cisor_ctx* c, const float2* f, const float2* w, float
 cisor_status grad_assemble(cisor_ctx* c, const float2* u, const float2* gz, const float2* s, double gamma,
                            float2* grad, float2* zstep, int ntx) {
   // the components of the vectorial model are consecutive [N] blocks of a transmitter: sum them too
-  grad_kernel<<<(unsigned)((c->N + 255) / 256), 256, 0, c->stream>>>(u, gz, ntx * c->ncomp, c->N, s, (float)gamma,
+  grad_kernel<<<(unsigned)((c->N + 31) / 32), 32 * GRAD_WARPS, 0, c->stream>>>(u, gz, ntx * c->ncomp, c->N, s, (float)gamma,
                                                                      c->complex_f, grad, zstep);
   CISOR_CUDA(cudaGetLastError());
   c->launches += 1;
