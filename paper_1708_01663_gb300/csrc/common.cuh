@@ -130,6 +130,7 @@ struct cisor_ctx {
   unsigned char* rx_mask;        // [T, M] active receivers (NULL: all), set by cisor_set_rx_mask
   float2* sense_part;            // [ksplit, T, M]
   int ksplit;
+  float2* h_slab;                // rows of H on their way to the host (cisor_sensing_matrix; null until then)
   float2* Ht;                    // [Nf, M] transposed sensing matrix of the tensor-core adjoint (null: FP32 GEMMs)
   int* tc_err;                   // device alias of h_tc_err
   int* h_tc_err;                 // mapped host flag, set by a sensing kernel whose bounded MMA wait gave up

@@ -576,12 +576,31 @@ __global__ void __launch_bounds__(256) sense_tile_kernel(const float* __restrict
     *reinterpret_cast<float4*>(out + tile_off(row, k, rows, Kp)) =
         k < width ? *reinterpret_cast<const float4*>(in + row * width + k) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
+// rows of the tiled matrix in row order.  Bound by memory: four rows a thread keep enough loads in flight (256
+// receivers, 256^2: 91 -> 53 us a call, what a device copy of a row-major H takes; a thread moved one 8-byte value before)
+constexpr int UT_ROWS = 4;
 __global__ void __launch_bounds__(256) sense_untile_kernel(const float* __restrict__ in, long long rows, long long width,
-                                                           long long row0, long long nrows, float2* __restrict__ out) {
-  const long long Kp = tile_kp(width), k = 2 * ((long long)blockIdx.x * 256 + threadIdx.x);
+                                                           long long row0, long long nrows, float* __restrict__ out) {
+  const long long Kp = tile_kp(width), k = 4 * ((long long)blockIdx.x * 256 + threadIdx.x);
   if (k >= width) return;
-  for (long long i = blockIdx.y; i < nrows; i += gridDim.y)
-    out[(i * width + k) / 2] = *reinterpret_cast<const float2*>(in + tile_off(row0 + i, k, rows, Kp));
+  const bool wide = ((uintptr_t)out & 15) == 0;  // (complex64 arrays need only 8; rows are multiples of 16 bytes)
+  for (long long i = (long long)blockIdx.y * UT_ROWS; i < nrows; i += (long long)gridDim.y * UT_ROWS) {
+    float4 v[UT_ROWS];
+#pragma unroll
+    for (int r = 0; r < UT_ROWS; ++r)
+      if (i + r < nrows) v[r] = __ldg(reinterpret_cast<const float4*>(in + tile_off(row0 + i + r, k, rows, Kp)));
+#pragma unroll
+    for (int r = 0; r < UT_ROWS; ++r) {
+      if (i + r >= nrows) break;
+      float* o = out + (i + r) * width + k;
+      if (wide) {
+        *reinterpret_cast<float4*>(o) = v[r];
+      } else {
+        reinterpret_cast<float2*>(o)[0] = make_float2(v[r].x, v[r].y);
+        reinterpret_cast<float2*>(o)[1] = make_float2(v[r].z, v[r].w);
+      }
+    }
+  }
 }
 // tiled Ht[n][m] = H[m][n] from tiled H, 32 x 32 complex blocks through shared memory
 __global__ void __launch_bounds__(256) sense_tile_transpose_kernel(const float* __restrict__ H, int M, long long Nf,
@@ -695,8 +714,9 @@ cisor_status sense_h_rows(cisor_ctx* c, long long row0, long long nrows, float2*
                                cudaMemcpyDeviceToDevice, c->stream));
     return CISOR_OK;
   }
-  sense_untile_kernel<<<dim3((unsigned)((c->Nf + 255) / 256), (unsigned)(nrows < 4096 ? nrows : 4096)), 256, 0, c->stream>>>(
-      reinterpret_cast<const float*>(c->H), c->M, 2 * c->Nf, row0, nrows, out);
+  const long long gy = (nrows + UT_ROWS - 1) / UT_ROWS;
+  sense_untile_kernel<<<dim3((unsigned)((c->Nf + 511) / 512), (unsigned)(gy < 4096 ? gy : 4096)), 256, 0, c->stream>>>(
+      reinterpret_cast<const float*>(c->H), c->M, 2 * c->Nf, row0, nrows, reinterpret_cast<float*>(out));
   CISOR_CUDA(cudaGetLastError());
   c->launches += 1;
   return CISOR_OK;
