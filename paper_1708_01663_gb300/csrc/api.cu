@@ -354,7 +354,7 @@ cisor_status cisor_create(cisor_ctx** out, const cisor_geometry* g, void* stream
   if (conv3_ok(d, P)) ALLOC(c->gplane, sizeof(float2) * conv3_ghat_elems(P));
   ALLOC(c->tw, sizeof(float2) * P);
   ALLOC(c->twst, sizeof(float2) * 2 * 512);
-  ALLOC(c->H, sense_h_bytes(c));
+  ALLOC(c->H, sense_h_bytes(c, c->M, c->Nf));
   ALLOC(c->u_in, TN);
   ALLOC(c->R, (size_t)c->T * c->ncomp * c->rtstride * sizeof(float2));
   ALLOC(c->r, TN);
@@ -379,7 +379,7 @@ cisor_status cisor_create(cisor_ctx** out, const cisor_geometry* g, void* stream
   {
     int ks = c->ksplit;
     if (sense_tc_ok(c)) {  // tensor-core sensing: the transposed matrix, the timeout flag, its split-K partials
-      ALLOC(c->Ht, sense_ht_bytes(c));
+      ALLOC(c->Ht, sense_h_bytes(c, c->Nf, c->M));
       cudaError_t e = cudaHostAlloc((void**)&c->h_tc_err, sizeof(int), cudaHostAllocMapped);
       if (e == cudaSuccess) {
         *c->h_tc_err = 0;

@@ -11,7 +11,7 @@
 //               the x and y FFTs; only the n non-zero z slabs are kept.
 //   ghat        [P^d]    complex64: spectrum of the circulant embedding of
 //               G (Sec. II, Eq. 3), pre-scaled by 1/P^d for the inverse FFTs
-//   H           [M, N]      complex64 (Eq. 2); as tiles where sense_tiled (sense_tc.cu)
+//   H           [M, N]      complex64 (Eq. 2); as tiles where sense_tiled (sense_tile.cuh)
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -347,9 +347,8 @@ cisor_status sense_adjoint(cisor_ctx* c, const float2* f, const float2* w, float
 bool sense_tc_ok(const cisor_ctx* c);
 int sense_tc_splits(const cisor_ctx* c, long long* KS);
 cisor_status sense_tc_setup(cisor_ctx* c);
-bool sense_tiled(const cisor_ctx* c);       // H and Ht are stored as tiles (sense_tc.cu)
-size_t sense_h_bytes(const cisor_ctx* c);
-size_t sense_ht_bytes(const cisor_ctx* c);
+bool sense_tiled(const cisor_ctx* c);       // H and Ht are stored as tiles (sense_tile.cuh)
+size_t sense_h_bytes(const cisor_ctx* c, long long rows, long long length);
 float2* sense_h_target(cisor_ctx* c);       // where the table kernels write H, row-major
 cisor_status sense_h_rows(cisor_ctx* c, long long row0, long long nrows, float2* out);
 cisor_status sense_tc_prepare(cisor_ctx* c);

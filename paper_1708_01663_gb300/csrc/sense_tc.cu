@@ -48,11 +48,11 @@
 // Every wait is bounded (a timeout sets the context's error flag, read by the host
 // after the call).
 #include "common.cuh"
+#include "sense_tile.cuh"
 #include "tc5.cuh"
 
 namespace cisor {
 
-constexpr int SK = 32;                       // K (floats) per chunk
 constexpr int SLBO = 144, SSBO = 8 * SLBO;   // K-group and 8-row strides of the operand tiles (bytes)
 constexpr int SPA = 16 * SSBO;               // bytes of one plane of the 128-row tile
 constexpr int STH = 256;                     // threads per CTA
@@ -66,15 +66,6 @@ constexpr long long S_MAX = 256;  // at most this many splits (partials T x M x 
 
 __host__ __device__ constexpr int soff(int row, int k) {
   return (row >> 3) * SSBO + (k >> 2) * SLBO + (row & 7) * 16 + (k & 3) * 4;
-}
-// float offset of (row, k) in a tiled [rows][Kp] matrix: tiles of 128 rows, chunks of SK floats within a tile (its
-// rows' 128 bytes one after another), 16-byte piece j of row r at j ^ (r % 8), so that 8 threads reading the same
-// piece of 8 rows from shared memory hit distinct banks.  Kp: the row length rounded up to SK (zeros behind it).
-__host__ __device__ __forceinline__ long long tile_kp(long long width) { return (width + SK - 1) / SK * SK; }
-__host__ __device__ __forceinline__ long long tile_off(long long row, long long k, long long rows, long long Kp) {
-  const long long r0 = row & ~127ll, R = rows - r0 < 128 ? rows - r0 : 128;
-  const int r = (int)(row - r0), j = (int)(k & (SK - 1)) >> 2;
-  return r0 * Kp + (k / SK) * (R * SK) + r * SK + ((j ^ (r & 7)) << 2) + (k & 3);
 }
 __device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
 __device__ __forceinline__ long long wrap(long long j, long long NP) {
@@ -272,9 +263,12 @@ constexpr int ws_smem(int nb) { return 1024 + SENSE_STAGES * WS_A + ws_dep(nb) *
 
 struct WsBars {
   uint64_t full[SENSE_STAGES], empty[SENSE_STAGES], ready[4], done[4];
+  int pieces[SENSE_STAGES];  // 16-byte pieces a row of the chunk in each load stage, where rows end in a narrow chunk
 };
 
-template <int ADJ, int NB>
+// NARROW: rows end in a chunk narrower than SK (tile_kp).  Compiled apart, since finding the chunk's width costs the
+// converters of every chunk: forward products of 64 transmitters, 256^2 36 -> 39 us with it, of one 23.4 -> 24.6.
+template <int ADJ, int NB, bool NARROW>
 __global__ void __launch_bounds__(ws_threads(NB), 1) sense_ws_kernel(const float* __restrict__ A, long long rows, int rtiles,
                                                             int nitems, long long K, long long KS,
                                                             const float2* __restrict__ src, long long lds,
@@ -350,11 +344,13 @@ __global__ void __launch_bounds__(ws_threads(NB), 1) sense_ws_kernel(const float
     for (uint32_t n = warp >> 2; n < total; n += GB) {
       const uint32_t s = n % SENSE_STAGES, buf = n % DEP, k = n / DEP;
       if (!wait_warp(&bar.full[s], n / SENSE_STAGES)) break;
-      const unsigned char* p = sm + s * WS_A + row * 128;  // (tile_off)
+      const int pieces = NARROW ? *(volatile int*)&bar.pieces[s] : SK / 4, z = tile_swz(row, pieces);
+      const unsigned char* p = sm + s * WS_A + row * pieces * 16;  // (tile_piece)
       uint32_t h[32], l[32];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const float4 x = *reinterpret_cast<const float4*>(p + ((j ^ (row & 7)) << 4));
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);  // behind the row's end, where B's zeros would not cancel an infinity
+        if (j < pieces) x = *reinterpret_cast<const float4*>(p + ((j ^ z) << 4));
         const float v[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -500,18 +496,20 @@ __global__ void __launch_bounds__(ws_threads(NB), 1) sense_ws_kernel(const float
     }
   } else if (warp == 16 + 4 * GB) {  // ---- producer
     if (lane == 0) {
-      const long long Kp = tile_kp(K);
+      const long long kp = tile_kp(K);
       uint32_t n = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
         const Item r = item(it);
-        const int R = rows - r.row0 < 128 ? (int)(rows - r.row0) : 128;  // (rows past the last keep old values)
-        const float* p = A + r.row0 * Kp + r.kb / SK * (R * SK);
+        const int R = tile_rows(r.row0, rows);  // (rows past the last keep old values)
+        const float* p = A + tile_chunk(r.row0, r.kb / SK, rows, kp);
         for (int ch = 0; ch < r.nch; ++ch, ++n, p += R * SK) {
           const uint32_t s = n % SENSE_STAGES;
           if (n >= SENSE_STAGES && !(ok = wait(&bar.empty[s], n / SENSE_STAGES - 1))) break;
-          mbar_expect(&bar.full[s], R * SK * 4);
-          bulk_load(sm + s * WS_A, p, R * SK * 4, &bar.full[s]);
+          const int w = NARROW ? tile_width(r.ke - r.kb - (long long)ch * SK) : SK;
+          if (NARROW) *(volatile int*)&bar.pieces[s] = w >> 2;
+          mbar_expect(&bar.full[s], R * w * 4);
+          bulk_load(sm + s * WS_A, p, R * w * 4, &bar.full[s]);
         }
       }
       // the loads still in flight land before the CTA's shared memory goes
@@ -570,10 +568,10 @@ __global__ void __launch_bounds__(256) sense_transpose_kernel(const float2* __re
 // row-major H [rows][width floats] into tiles, and back; a thread moves 16 bytes (zeros behind the row's end)
 __global__ void __launch_bounds__(256) sense_tile_kernel(const float* __restrict__ in, long long rows, long long width,
                                                          float* __restrict__ out) {
-  const long long Kp = tile_kp(width), k = 4 * ((long long)blockIdx.x * 256 + threadIdx.x);
-  if (k >= Kp) return;
+  const long long kp = tile_kp(width), k = 4 * ((long long)blockIdx.x * 256 + threadIdx.x);
+  if (k >= kp) return;
   for (long long row = blockIdx.y; row < rows; row += gridDim.y)
-    *reinterpret_cast<float4*>(out + tile_off(row, k, rows, Kp)) =
+    *reinterpret_cast<float4*>(out + tile_off(row, k, rows, kp)) =
         k < width ? *reinterpret_cast<const float4*>(in + row * width + k) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 // rows of the tiled matrix in row order.  Bound by memory: four rows a thread keep enough loads in flight (256
@@ -581,14 +579,14 @@ __global__ void __launch_bounds__(256) sense_tile_kernel(const float* __restrict
 constexpr int UT_ROWS = 4;
 __global__ void __launch_bounds__(256) sense_untile_kernel(const float* __restrict__ in, long long rows, long long width,
                                                            long long row0, long long nrows, float* __restrict__ out) {
-  const long long Kp = tile_kp(width), k = 4 * ((long long)blockIdx.x * 256 + threadIdx.x);
+  const long long kp = tile_kp(width), k = 4 * ((long long)blockIdx.x * 256 + threadIdx.x);
   if (k >= width) return;
   const bool wide = ((uintptr_t)out & 15) == 0;  // (complex64 arrays need only 8; rows are multiples of 16 bytes)
   for (long long i = (long long)blockIdx.y * UT_ROWS; i < nrows; i += (long long)gridDim.y * UT_ROWS) {
     float4 v[UT_ROWS];
 #pragma unroll
     for (int r = 0; r < UT_ROWS; ++r)
-      if (i + r < nrows) v[r] = __ldg(reinterpret_cast<const float4*>(in + tile_off(row0 + i + r, k, rows, Kp)));
+      if (i + r < nrows) v[r] = __ldg(reinterpret_cast<const float4*>(in + tile_off(row0 + i + r, k, rows, kp)));
 #pragma unroll
     for (int r = 0; r < UT_ROWS; ++r) {
       if (i + r >= nrows) break;
@@ -606,19 +604,19 @@ __global__ void __launch_bounds__(256) sense_untile_kernel(const float* __restri
 __global__ void __launch_bounds__(256) sense_tile_transpose_kernel(const float* __restrict__ H, int M, long long Nf,
                                                                    float* __restrict__ Ht) {
   __shared__ float2 tile[32][33];
-  const long long n0 = (long long)blockIdx.x * 32, Kh = tile_kp(2 * Nf), Kt = tile_kp(2 * (long long)M);
+  const long long n0 = (long long)blockIdx.x * 32, kh = tile_kp(2 * Nf), kt = tile_kp(2 * (long long)M);
   const int m0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   for (int i = ty; i < 32; i += 8) {
     const int m = m0 + i;
     const long long n = n0 + tx;
-    tile[i][tx] = m < M && n < Nf ? *reinterpret_cast<const float2*>(H + tile_off(m, 2 * n, M, Kh)) : make_float2(0.f, 0.f);
+    tile[i][tx] = m < M && n < Nf ? *reinterpret_cast<const float2*>(H + tile_off(m, 2 * n, M, kh)) : make_float2(0.f, 0.f);
   }
   __syncthreads();
   for (int i = ty; i < 32; i += 8) {
     const long long n = n0 + i;
     const int m = m0 + tx;
-    if (2 * m < Kt && n < Nf) *reinterpret_cast<float2*>(Ht + tile_off(n, 2 * (long long)m, Nf, Kt)) = tile[tx][i];
+    if (2 * m < kt && n < Nf) *reinterpret_cast<float2*>(Ht + tile_off(n, 2 * m, Nf, kt)) = tile[tx][i];
   }
 }
 
@@ -628,26 +626,28 @@ bool sense_tc_ok(const cisor_ctx* c) {
   return c->T <= 128 && c->Nf % 2 == 0 && c->M % 2 == 0;
 }
 bool sense_tiled(const cisor_ctx* c) { return sense_tc_ok(c) && sense_tc_cols(c->T) <= WS_NB; }
-size_t sense_h_bytes(const cisor_ctx* c) {
-  return sense_tiled(c) ? sizeof(float) * (size_t)(c->M * tile_kp(2 * c->Nf)) : sizeof(float2) * (size_t)c->M * c->Nf;
-}
-size_t sense_ht_bytes(const cisor_ctx* c) {
-  return sense_tiled(c) ? sizeof(float) * (size_t)(c->Nf * tile_kp(2 * (long long)c->M)) : sizeof(float2) * (size_t)c->M * c->Nf;
+// bytes of H (rows = M of length Nf) or Ht (the other way round)
+size_t sense_h_bytes(const cisor_ctx* c, long long rows, long long length) {
+  return sense_tiled(c) ? sizeof(float) * (size_t)(rows * tile_kp(2 * length)) : sizeof(float2) * (size_t)rows * length;
 }
 
 // the warp-specialised kernel for nb <= 192 accumulator columns (sense_tc_cols)
-template <int ADJ>
 using ws_fn = void (*)(const float*, long long, int, int, long long, long long, const float2*, long long, const float2*,
                        long long, int, int, long long, float2*, float2*, int*);
-template <int ADJ>
-ws_fn<ADJ> ws_kernel_for(int nb) {
+template <int ADJ, bool NARROW>
+static ws_fn ws_kernel_of(int nb) {
   switch (nb) {
-    case 32: return sense_ws_kernel<ADJ, 32>;
-    case 64: return sense_ws_kernel<ADJ, 64>;
-    case 96: return sense_ws_kernel<ADJ, 96>;
-    case 128: return sense_ws_kernel<ADJ, 128>;
-    default: return sense_ws_kernel<ADJ, 192>;
+    case 32: return sense_ws_kernel<ADJ, 32, NARROW>;
+    case 64: return sense_ws_kernel<ADJ, 64, NARROW>;
+    case 96: return sense_ws_kernel<ADJ, 96, NARROW>;
+    case 128: return sense_ws_kernel<ADJ, 128, NARROW>;
+    default: return sense_ws_kernel<ADJ, 192, NARROW>;
   }
+}
+// for rows of K floats
+template <int ADJ>
+static ws_fn ws_kernel_for(int nb, long long K) {
+  return tile_kp(K) % SK ? ws_kernel_of<ADJ, true>(nb) : ws_kernel_of<ADJ, false>(nb);
 }
 
 // kernel attributes (shared memory, carveout) and, for more transmitters than the warp-specialised kernel takes, the
@@ -656,7 +656,7 @@ cisor_status sense_tc_setup(cisor_ctx* c) {
   const int nb = sense_tc_cols(c->T);
   c->sense_tc_occ = 1;
   if (sense_tiled(c)) {
-    for (const void* fn : {(const void*)ws_kernel_for<0>(nb), (const void*)ws_kernel_for<1>(nb)})
+    for (const void* fn : {(const void*)ws_kernel_for<0>(nb, 2 * c->Nf), (const void*)ws_kernel_for<1>(nb, 2 * (long long)c->M)})
       CISOR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ws_smem(nb)));
     return CISOR_OK;
   }
@@ -691,9 +691,8 @@ int sense_tc_splits(const cisor_ctx* c, long long* KS) {
 float2* sense_h_target(cisor_ctx* c) { return sense_tiled(c) ? c->Ht : c->H; }
 cisor_status sense_tc_prepare(cisor_ctx* c) {
   if (!c->Ht) return CISOR_OK;
-  const long long Kh = tile_kp(2 * c->Nf);
   if (sense_tiled(c)) {
-    sense_tile_kernel<<<dim3((unsigned)((Kh / 4 + 255) / 256), (unsigned)(c->M < 4096 ? c->M : 4096)), 256, 0, c->stream>>>(
+    sense_tile_kernel<<<dim3((unsigned)((tile_kp(2 * c->Nf) / 4 + 255) / 256), (unsigned)(c->M < 4096 ? c->M : 4096)), 256, 0, c->stream>>>(
         reinterpret_cast<const float*>(c->Ht), c->M, 2 * c->Nf, reinterpret_cast<float*>(c->H));
     CISOR_CUDA(cudaGetLastError());
     const dim3 g((unsigned)((c->Nf + 31) / 32), (unsigned)((tile_kp(2 * (long long)c->M) / 2 + 31) / 32));
@@ -732,7 +731,7 @@ static cisor_status sense_tc_gemm(cisor_ctx* c, long long rows, long long K, lon
   const float* A = reinterpret_cast<const float*>(ADJ ? c->Ht : c->H);
   if (sense_tiled(c)) {
     const int nb = sense_tc_cols(c->T), nitems = rtiles * splits;  // (the attributes were set for T's width)
-    ws_kernel_for<ADJ>(nb)<<<nitems < c->sms ? nitems : c->sms, ws_threads(nb), ws_smem(nb), c->stream>>>(
+    ws_kernel_for<ADJ>(nb, K)<<<nitems < c->sms ? nitems : c->sms, ws_threads(nb), ws_smem(nb), c->stream>>>(
         A, rows, rtiles, nitems, K, KS, src, lds, f, c->N, ntx, c->M, c->Nf,
         out0, out1, c->tc_err);
   } else {
