@@ -15,6 +15,8 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include "sense_tile.cuh"
 #include <string>
 #include <vector>
 
@@ -349,7 +351,25 @@ int sense_tc_splits(const cisor_ctx* c, long long* KS);
 cisor_status sense_tc_setup(cisor_ctx* c);
 bool sense_tiled(const cisor_ctx* c);       // H and Ht are stored as tiles (sense_tile.cuh)
 size_t sense_h_bytes(const cisor_ctx* c, long long rows, long long length);
-float2* sense_h_target(cisor_ctx* c);       // where the table kernels write H, row-major
+// H as the table kernels write it: row-major (kp = 0), or as tiles with their zeros behind a row's end, which costs
+// nothing beside the FP64 evaluation of an entry (a pass of its own over 1024 receivers, 64^3 took 0.9 ms of 41)
+struct SenseTable {
+  float2* H;
+  long long rows, length, kp;
+#ifdef __CUDACC__
+  __device__ __forceinline__ void store(long long m, long long n, float2 v) const {
+    if (!kp) {
+      H[m * length + n] = v;
+      return;
+    }
+    float* h = reinterpret_cast<float*>(H);
+    *reinterpret_cast<float2*>(h + tile_off(m, 2 * n, rows, kp)) = v;
+    if (n == length - 1)
+      for (long long k = 2 * length; k < kp; k += 2) *reinterpret_cast<float2*>(h + tile_off(m, k, rows, kp)) = make_float2(0.f, 0.f);
+  }
+#endif
+};
+SenseTable sense_table(const cisor_ctx* c);
 cisor_status sense_h_rows(cisor_ctx* c, long long row0, long long nrows, float2* out);
 cisor_status sense_tc_prepare(cisor_ctx* c);
 cisor_status sense_tc_forward(cisor_ctx* c, const float2* f, const float2* u, int ntx, int* splits);

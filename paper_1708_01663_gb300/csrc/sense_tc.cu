@@ -565,15 +565,6 @@ __global__ void __launch_bounds__(256) sense_transpose_kernel(const float2* __re
   }
 }
 
-// row-major H [rows][width floats] into tiles, and back; a thread moves 16 bytes (zeros behind the row's end)
-__global__ void __launch_bounds__(256) sense_tile_kernel(const float* __restrict__ in, long long rows, long long width,
-                                                         float* __restrict__ out) {
-  const long long kp = tile_kp(width), k = 4 * ((long long)blockIdx.x * 256 + threadIdx.x);
-  if (k >= kp) return;
-  for (long long row = blockIdx.y; row < rows; row += gridDim.y)
-    *reinterpret_cast<float4*>(out + tile_off(row, k, rows, kp)) =
-        k < width ? *reinterpret_cast<const float4*>(in + row * width + k) : make_float4(0.f, 0.f, 0.f, 0.f);
-}
 // rows of the tiled matrix in row order.  Bound by memory: four rows a thread keep enough loads in flight (256
 // receivers, 256^2: 91 -> 53 us a call, what a device copy of a row-major H takes; a thread moved one 8-byte value before)
 constexpr int UT_ROWS = 4;
@@ -687,14 +678,11 @@ int sense_tc_splits(const cisor_ctx* c, long long* KS) {
   return (int)((K + ks - 1) / ks);
 }
 
-// H, written row-major into sense_h_target(c) by the table kernels, into its final place and form, and Ht from it
-float2* sense_h_target(cisor_ctx* c) { return sense_tiled(c) ? c->Ht : c->H; }
+SenseTable sense_table(const cisor_ctx* c) { return {c->H, c->M, c->Nf, sense_tiled(c) ? tile_kp(2 * c->Nf) : 0}; }
+// Ht from H
 cisor_status sense_tc_prepare(cisor_ctx* c) {
   if (!c->Ht) return CISOR_OK;
   if (sense_tiled(c)) {
-    sense_tile_kernel<<<dim3((unsigned)((tile_kp(2 * c->Nf) / 4 + 255) / 256), (unsigned)(c->M < 4096 ? c->M : 4096)), 256, 0, c->stream>>>(
-        reinterpret_cast<const float*>(c->Ht), c->M, 2 * c->Nf, reinterpret_cast<float*>(c->H));
-    CISOR_CUDA(cudaGetLastError());
     const dim3 g((unsigned)((c->Nf + 31) / 32), (unsigned)((tile_kp(2 * (long long)c->M) / 2 + 31) / 32));
     sense_tile_transpose_kernel<<<g, 256, 0, c->stream>>>(reinterpret_cast<const float*>(c->H), c->M, c->Nf,
                                                           reinterpret_cast<float*>(c->Ht));

@@ -152,7 +152,7 @@ __global__ void fft64_cols_kernel(double2* data, const double2* tw_g, size_t es,
   }
 }
 
-__global__ void sensing_kernel(float2* H, const double* rx, int M, int n, double delta, double k, double kb) {
+__global__ void sensing_kernel(const SenseTable H, const double* rx, int M, int n, double delta, double k, double kb) {
   long long N = (long long)n * n;
   long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)M * N) return;
@@ -162,10 +162,10 @@ __global__ void sensing_kernel(float2* H, const double* rx, int M, int n, double
   double x = (ix - n / 2.0 + 0.5) * delta, y = (iy - n / 2.0 + 0.5) * delta;
   double dx = rx[2 * m] - x, dy = rx[2 * m + 1] - y;
   double2 g = green2d_scaled(sqrt(dx * dx + dy * dy), k, kb, delta);
-  H[idx] = make_float2((float)g.x, (float)g.y);
+  H.store(m, p, make_float2((float)g.x, (float)g.y));
 }
 
-__global__ void sensing3d_kernel(float2* H, const double* rx, int M, int n, double delta, double k, double kb) {
+__global__ void sensing3d_kernel(const SenseTable H, const double* rx, int M, int n, double delta, double k, double kb) {
   const long long N = (long long)n * n * n;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)M * N) return;
@@ -176,7 +176,7 @@ __global__ void sensing3d_kernel(float2* H, const double* rx, int M, int n, doub
   const double dx = rx[3 * m] - (ix - h) * delta, dy = rx[3 * m + 1] - (iy - h) * delta,
                dz = rx[3 * m + 2] - (iz - h) * delta;
   const double2 g = green3d_scaled(sqrt(dx * dx + dy * dy + dz * dz), k, kb, delta);
-  H[idx] = make_float2((float)g.x, (float)g.y);
+  H.store(m, p, make_float2((float)g.x, (float)g.y));
 }
 
 // exp(j kb d_t . r) for unit directions d_t (3D plane waves)
@@ -336,9 +336,9 @@ cisor_status build_tables(cisor_ctx* c) {
   if (c->ncomp == 3) {  // vectorial model: dyadic sensing row and polarised plane waves
     CISOR_TRY(vec_tables(c, d_ang, d_rx));
   } else if (d == 3)
-    sensing3d_kernel<<<(unsigned)((MN + 255) / 256), 256, 0, c->stream>>>(sense_h_target(c), d_rx, c->M, n, c->delta, c->k, c->kb);
+    sensing3d_kernel<<<(unsigned)((MN + 255) / 256), 256, 0, c->stream>>>(sense_table(c), d_rx, c->M, n, c->delta, c->k, c->kb);
   else
-    sensing_kernel<<<(unsigned)((MN + 255) / 256), 256, 0, c->stream>>>(sense_h_target(c), d_rx, c->M, n, c->delta, c->k, c->kb);
+    sensing_kernel<<<(unsigned)((MN + 255) / 256), 256, 0, c->stream>>>(sense_table(c), d_rx, c->M, n, c->delta, c->k, c->kb);
   CISOR_CUDA(cudaGetLastError());
   CISOR_TRY(sense_tc_prepare(c));
   const unsigned gT = (unsigned)((TN + 255) / 256);

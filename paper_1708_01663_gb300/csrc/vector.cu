@@ -310,7 +310,7 @@ cisor_status vec_axpy(cisor_ctx* c, int ntx) {
 }
 
 // ---------------------------------------------------------------- tables (FP64)
-__global__ void dyadic_sensing_kernel(float2* H, const double* rx, int M, int n, double delta, double k) {
+__global__ void dyadic_sensing_kernel(const SenseTable H, const double* rx, int M, int n, double delta, double k) {
   const long long N = (long long)n * n * n, K = 3 * N;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)M * K) return;
@@ -335,7 +335,7 @@ __global__ void dyadic_sensing_kernel(float2* H, const double* rx, int M, int n,
   if (c == 2) coef = z_add(coef, bv);
   const double s = k * k * delta * delta * delta;
   const double2 v = z_mul(coef, g);
-  H[idx] = make_float2((float)(s * v.x), (float)(s * v.y));
+  H.store(m, rem, make_float2((float)(s * v.x), (float)(s * v.y)));
 }
 
 __global__ void polarised_wave_kernel(float2* u, const double* tx, int T, int n, double delta, double k) {
@@ -358,7 +358,7 @@ __global__ void polarised_wave_kernel(float2* u, const double* tx, int T, int n,
 
 cisor_status vec_tables(cisor_ctx* c, const double* d_tx, const double* d_rx) {
   const long long MK = (long long)c->M * c->Nf, TK = (long long)c->T * c->Nf;
-  dyadic_sensing_kernel<<<(unsigned)((MK + 255) / 256), 256, 0, c->stream>>>(sense_h_target(c), d_rx, c->M, c->n, c->delta, c->k);
+  dyadic_sensing_kernel<<<(unsigned)((MK + 255) / 256), 256, 0, c->stream>>>(sense_table(c), d_rx, c->M, c->n, c->delta, c->k);
   CISOR_CUDA(cudaGetLastError());
   polarised_wave_kernel<<<(unsigned)((TK + 255) / 256), 256, 0, c->stream>>>(c->u_in, d_tx, c->T, c->n, c->delta, c->k);
   CISOR_CUDA(cudaGetLastError());
