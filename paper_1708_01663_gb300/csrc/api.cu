@@ -220,11 +220,16 @@ static void free_ctx(cisor_ctx* c) {
 
 static bool two_stage_ok(const cisor_ctx* c) { return c->P == 128 || c->P == 256 || (c->dim == 2 && c->P == 512); }
 
-// Column shape of a context until it is set or autotuned, from back-to-back passes on 1 to 64 transmitters.  P = 512
+// Column shape of a context until it is set or autotuned, from back-to-back passes on 1 to 64 transmitters.  2D, P = 512
 // and 256: two-stage (64 transmitters 90 against 107 and 126 us with 512 and 256 threads; P = 256: 23 against 28 us;
 // one transmitter: 12 against 13 us).  P <= 128: 256 threads, whose smaller CTAs suit the few columns there are (P =
 // 128, 8 transmitters: 7.9 against 9.1 us with 512 threads, 64 of them: 12.8 against 13.2; P = 64: 6.3 against 7.0).
-static int default_shape(const cisor_ctx* c) { return c->P >= 256 && two_stage_ok(c) ? COLS_TWO_STAGE : 256; }
+// 3D, P = 256: 512 threads (65^3 to 128^3, 1 to 8 transmitters: two-stage columns 9 to 20 % slower, 72^3 102 against 120
+// us; 256 threads, whose twiddles are products, 6 to 9 % faster, which is left to the autotuner).
+static int default_shape(const cisor_ctx* c) {
+  if (c->dim == 3) return c->P == 256 ? 512 : 256;
+  return c->P >= 256 ? COLS_TWO_STAGE : 256;
+}
 
 }  // namespace cisor
 

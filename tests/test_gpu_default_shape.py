@@ -1,0 +1,39 @@
+"""The column shape that a context starts with, and 3D passes with P = 256 for every shape that the autotuner can pick."""
+import numpy as np
+import pytest
+
+from oracle import model
+from paper_1708_01663_gb300 import build, cisor, synth
+from tests.gpu_util import c64, rel
+
+pytestmark = pytest.mark.gpu
+DELTA = 1.0 / 6
+
+
+@pytest.mark.parametrize("dim,n,pad,shape", [(2, 20, 0, 256), (2, 64, 0, 256), (2, 65, 0, 16), (2, 129, 0, 16), (3, 20, 0, 256),
+                                             (3, 20, 256, 512)])
+def test_default(dim, n, pad, shape):
+    build.build()
+    if dim == 2:
+        ctx = cisor.Cisor(n, DELTA, synth.plane_wave_angles(2), synth.circle_receivers(4, DELTA * n), pad=pad)
+    else:
+        ctx = cisor.Cisor(n, DELTA, synth.hemisphere_directions()[:2], synth.planar_receivers(2, 0.5, DELTA * n), dim=3, pad=pad)
+    assert ctx.tuning() == (shape, 0)
+
+
+@pytest.mark.parametrize("shape", [512, 256, 16])
+@pytest.mark.parametrize("n", [20, 33])
+def test_columns_3d_p256(n, shape):
+    """y forward, z with the spectrum, y back: A x and A^H x against the oracle (2e-5, the matvec's tolerance)."""
+    build.build()
+    dirs, rx = synth.hemisphere_directions()[:2], synth.planar_receivers(2, 0.5, DELTA * n)
+    ctx = cisor.Cisor(n, DELTA, dirs, rx, complex_f=True, dim=3, pad=256)
+    prob = model.Problem(n, DELTA, dirs, rx, P=256, dim=3)
+    ctx.set_cols_cta(shape)
+    f = synth.sphere_phantom(n, 4, (0.0, 0.6), 7, imag=0.05)
+    x = synth.random_field(8, (2, n, n, n))
+    y = np.empty((2, n, n, n), np.complex64)
+    for adjoint, op in ((False, prob.A), (True, prob.AH)):
+        ctx.apply_A(c64(f), c64(x), y, adjoint=adjoint)
+        for t in range(2):
+            assert rel(y[t], op(c64(f).astype(np.complex128), x[t])) < 2e-5
