@@ -325,6 +325,7 @@ cisor_status cisor_create(cisor_ctx** out, const cisor_geometry* g, void* stream
   c->graph_chunk = 4;
   c->use_while = 0;  // host-driven chunks by default: profilers list the kernels of these graphs
   c->cols_nt = default_shape(c);
+  c->cols_auto = 1;
   conv_geometry(c);
   {
     // split-K of the forward sensing GEMM: about 4 CTAs per SM, chunks of >= 256 pixels
@@ -853,8 +854,9 @@ cisor_status cisor_set_cols_cta(cisor_ctx* c, int cols_nt) {
               "(this grid: %dD, P = %d)", COLS_TWO_STAGE, c->dim, c->P);
     return CISOR_ERR_INVALID_ARG;
   }
-  if (cols_nt != c->cols_nt) {
+  if (cols_nt != c->cols_nt || c->cols_auto) {
     c->cols_nt = cols_nt;
+    c->cols_auto = 0;
     CISOR_TRY(drop_graphs(c));
   }
   return CISOR_OK;
@@ -933,6 +935,7 @@ cisor_status cisor_autotune(cisor_ctx* c, int reps, int* cols_nt_out) {
     const long long k = ((long long)mb << 20) / rbytes;
     if (k >= 1 && k < ntr && (nch == 1 || k != chunks[nch - 1])) chunks[nch++] = (int)k;
   }
+  c->cols_auto = 0;
   int best = variants[0], best_chunk = 0;
   float best_ms = 1e30f;
   cisor_status st = CISOR_OK;

@@ -168,6 +168,7 @@ struct cisor_ctx {
   long long launches;       // kernels launched (graph replays add their kernel count)
   int cols_nt;              // column-FFT kernel shape (512 or 256 threads of the three-stage kernel, or
                             // COLS_TWO_STAGE), set by the autotuner
+  int cols_auto;            // cols_nt is still the default by size (cols_shape refines it)
   int tx_chunk;             // transforms per convolution launch (0: all at once); every chunk reuses the
                             // start of R, so a chunk's intermediate can stay in L2 between its kernels
   long long graph_kernels[2];

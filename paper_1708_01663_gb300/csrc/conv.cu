@@ -535,16 +535,29 @@ static void launch_cols_2s(cisor_ctx* c, const ConvOp& op, int nslab, long long 
   }
 }
 
+// The column shape of one pass: the context's.  Until that is set or autotuned, fewer than six transforms at P = 512
+// take 512 threads instead of the two-stage kernel, whose 32 CTAs a transform leave most SMs idle while each works
+// longer: an iteration of a solve takes 41.1, 49.3 and 49.2 us with one, four and five transmitters at 129^2 against
+// 45.2, 53.0 and 52.9, at 256^2 41.6, 54.1, 57.2 against 46.0, 55.8, 59.6 (two transmitters within 3 % either way; six
+// are faster with the two-stage kernel, 61.8 against 64.1, seven vary by size, eight 65.1 against 71).  A single
+// transform outside an iteration keeps the two-stage kernel: 11.8 against 13.1 us a pass at 256^2, equal at 129^2.
+template <int P>
+static int cols_shape(const cisor_ctx* c, const ConvOp& op) {
+  if (P != 512 || !c->cols_auto || op.ntx >= 6 || (op.ntx == 1 && !op.active)) return c->cols_nt;
+  return 512;
+}
+
 template <int P, int MODE>
 static void cols_pass(cisor_ctx* c, const ConvOp& op, int nslab, long long es, long long slab) {
-  if (c->cols_nt == COLS_TWO_STAGE || c->cols_nt == COLS_CLUSTER) {  // (combinations the cluster pass lacks)
+  const int shape = cols_shape<P>(c, op);
+  if (shape == COLS_TWO_STAGE || shape == COLS_CLUSTER) {  // (combinations the cluster pass lacks)
     if (op.adjoint)
       launch_cols_2s<P, MODE, true>(c, op, nslab, es, slab);
     else
       launch_cols_2s<P, MODE, false>(c, op, nslab, es, slab);
     return;
   }
-  if (c->cols_nt == 256) {
+  if (shape == 256) {
     if (op.adjoint)
       launch_cols<P, MODE, true, 256>(c, op, nslab, es, slab);
     else
