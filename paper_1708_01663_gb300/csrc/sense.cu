@@ -16,6 +16,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "fp32_sum.cuh"
 
 namespace cisor {
 
@@ -113,59 +114,54 @@ __global__ void __launch_bounds__(256, 2) sense_fwd_kernel(const float2* __restr
     }
 }
 
-// s + e += p with the rounding error of every sum kept in e (Knuth's TwoSum)
-__device__ __forceinline__ void two_sum(float& s, float& e, float p) {
-  const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
-  e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b)));
-  s = t;
-}
-
 // Z = sum of the ks split-K partials, w = Z - y (0 at receivers a transmitter does not record), and
 // D += 1/2 sum |w|^2.  A CTA takes 32 consecutive entries (lanes, coalesced); its 8 warps sum the partials
-// k = w, w + 8, ... and warp 0 adds the 8 sums in FP64 in warp order (the same order every call).  A warp sums its
-// partials as pairs of FP32 values (two_sum: 48 bits), since FP64 runs at a small fraction of the FP32 rate: 256
-// partials of 48 x 1024 entries cost 78 us more by FP64 additions (1265 -> 1185 us for both sensing products).  A sum that is not finite is taken again in FP64.
+// k = w, w + 8, ... and warp 0 adds the 8 sums in warp order (the same order every call).  All of it in three FP32
+// values a sum and one conversion an entry (fp32_sum.cuh: no less exact than FP64, which runs at a small fraction of
+// the FP32 rate: 256 splits of 48 x 1024 entries 671 -> 593 us for the product, 147 of 64 x 256 76 -> 67, this kernel
+// 15 -> 7 us there).  A sum that is not finite is taken again in FP64, whose range is wider.  Four partials a step: eight
+// or two are 0.5 to 1 us slower where a warp has six.
 constexpr int RED_WARPS = 8;
 __global__ void __launch_bounds__(32 * RED_WARPS) sense_reduce_kernel(const float2* __restrict__ part, int ks, int T,
                                                                      int M, const float2* __restrict__ y,
                                                                      float2* __restrict__ Z, float2* __restrict__ w,
                                                                      double* __restrict__ dsum,
                                                                      const unsigned char* __restrict__ mask) {
-  __shared__ double2 red[RED_WARPS][32];
+  __shared__ float red[RED_WARPS][6][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int idx = blockIdx.x * 32 + lane;
   const long long TM = (long long)T * M;
-  double sx = 0.0, sy = 0.0;
+  Fp32Sum a, b;  // real and imaginary parts
   if (idx < TM) {
-    float2 s = make_float2(0.f, 0.f), e = make_float2(0.f, 0.f);
-#pragma unroll 8
+#pragma unroll 4
     for (int k = warp; k < ks; k += RED_WARPS) {
       const float2 p = part[(long long)k * TM + idx];
-      two_sum(s.x, e.x, p.x);
-      two_sum(s.y, e.y, p.y);
-    }
-    sx = (double)s.x + (double)e.x;
-    sy = (double)s.y + (double)e.y;
-    if (!isfinite(e.x) || !isfinite(e.y)) {
-      sx = sy = 0.0;
-      for (int k = warp; k < ks; k += RED_WARPS) {
-        const float2 p = part[(long long)k * TM + idx];
-        sx += p.x;
-        sy += p.y;
-      }
+      a.add(p.x);
+      b.add(p.y);
     }
   }
-  red[warp][lane] = make_double2(sx, sy);
+  const float own[6] = {a.s, a.e, a.c, b.s, b.e, b.c};
+#pragma unroll
+  for (int j = 0; j < 6; ++j) red[warp][j][lane] = own[j];
   __syncthreads();
   if (warp != 0) return;
   double d = 0.0;
   if (idx < TM) {
-    sx = 0.0;
-    sy = 0.0;
 #pragma unroll
-    for (int i = 0; i < RED_WARPS; ++i) {
-      sx += red[i][lane].x;
-      sy += red[i][lane].y;
+    for (int i = 1; i < RED_WARPS; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        a.add(red[i][j][lane]);
+        b.add(red[i][3 + j][lane]);
+      }
+    double sx = a.value(), sy = b.value();
+    if (!isfinite(sx) || !isfinite(sy)) {
+      sx = sy = 0.0;
+      for (int k = 0; k < ks; ++k) {
+        const float2 p = part[(long long)k * TM + idx];
+        sx += p.x;
+        sy += p.y;
+      }
     }
     if (Z) Z[idx] = make_float2((float)sx, (float)sy);
     if (y) {
