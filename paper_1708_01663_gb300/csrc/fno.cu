@@ -191,14 +191,9 @@ __device__ __forceinline__ void load_planar(float* dst, const float* src, int b,
     cp16(dst + c * NPP + 4 * q, src + ((long long)b * FC + c) * FNN + pix0 + 4 * q);
   }
 }
-// a 32 x 32 BF16 weight matrix W[o][i] into shared memory, as Ws[o][i] (pitch WP) and / or Wt[i][o]
-__device__ __forceinline__ void load_w(const __nv_bfloat16* __restrict__ w, __nv_bfloat16* ws, __nv_bfloat16* wt) {
-  for (int e = threadIdx.x; e < FC * FC; e += NTH) {
-    const int o = e / FC, i = e % FC;
-    const __nv_bfloat16 v = w[e];
-    if (ws) ws[o * WP + i] = v;
-    if (wt) wt[i * WP + o] = v;
-  }
+// a 32 x 32 BF16 weight matrix W[o][i] into shared memory, transposed (pitch WP)
+__device__ __forceinline__ void load_wt(const __nv_bfloat16* __restrict__ w, __nv_bfloat16* wt) {
+  for (int e = threadIdx.x; e < FC * FC; e += NTH) wt[(e % FC) * WP + e / FC] = w[e];
 }
 
 // ------------------------------------------------------------------ shared phases of the row kernels
@@ -211,8 +206,8 @@ __device__ __forceinline__ const uint32_t* tab_ri(const __nv_bfloat16* tb, int l
 
 // S(rr, ix) = Re sum_ky Z[ky][c][r] exp(+2 pi j ky ix / 128), rr = 32 r + c: GEMM
 // M = 64 (rr), N = 128 (ix), K = 32 (Re / Im of the 16 ky).  Adds into
-// dst[c * NPP + r * FN + ix] (accumulate) or stores there.
-__device__ __forceinline__ void row_inverse(const float2* zs, const __nv_bfloat16* tb, float* dst, bool accumulate) {
+// dst[c * NPP + r * FN + ix].
+__device__ __forceinline__ void row_inverse(const float2* zs, const __nv_bfloat16* tb, float* dst) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const float* zf = reinterpret_cast<const float*>(zs);
   auto A = [&](int rr, int k) { return zf[(((k >> 1) * FC + (rr & 31)) * RB + (rr >> 5)) * 2 + (k & 1)]; };
@@ -237,8 +232,7 @@ __device__ __forceinline__ void row_inverse(const float2* zs, const __nv_bfloat1
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int rr = 16 * mt + g + (e >> 1) * 8, ix = 8 * (nt0 + j) + 2 * t + (e & 1);
-      float* p = dst + (rr & 31) * NPP + (rr >> 5) * FN + ix;
-      *p = accumulate ? *p + d[j][e] : d[j][e];
+      dst[(rr & 31) * NPP + (rr >> 5) * FN + ix] += d[j][e];
     }
 }
 
@@ -268,30 +262,6 @@ __device__ __forceinline__ void row_forward(const float* src, const __nv_bfloat1
       const int rr = 16 * mt + g + 8 * h, ky = 4 * (nt0 + j) + t;
       stage[(ky * FC + (rr & 31)) * RB + (rr >> 5)] = make_float2(d[j][2 * h], d[j][2 * h + 1]);
     }
-}
-
-// out[p][o] (+)= sum_i A(p, i) W[o][i] over the NP pixels (M = NP, N = FC, K = FC), W exact BF16 in
-// ws ([o][i], pitch WP); epi(p, o, value) consumes each result once.
-template <class FA, class Epi>
-__device__ __forceinline__ void pixel_mix(FA A, const __nv_bfloat16* ws, Epi epi) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-  const uint32_t* w32 = reinterpret_cast<const uint32_t*>(ws);
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int mt = 2 * warp + h;
-    const FragA a0 = load_a(A, 16 * mt, 0, g, t), a1 = load_a(A, 16 * mt, 16, g, t);
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      uint32_t b0[2], b1[2];
-      load_b_tab(w32, WP / 2, 0, 8 * nt, g, t, b0);
-      load_b_tab(w32, WP / 2, 16, 8 * nt, g, t, b1);
-      float d[4] = {0.f, 0.f, 0.f, 0.f};
-      mma2(d, a0, b0);
-      mma2(d, a1, b1);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) epi(16 * mt + g + (e >> 1) * 8, 8 * nt + 2 * t + (e & 1), d[e]);
-    }
-  }
 }
 
 // the 8 input features of the NP pixels of rows iy0, iy0 + 1 into as[k * NPP + p]
@@ -976,7 +946,7 @@ __global__ void __launch_bounds__(NTH, 2) fno_row_bwd(const float* __restrict__ 
   const int j8 = lane >> 3, l8 = lane & 7;  // ldmatrix: this lane's matrix and row
   pdl_trigger();
   cta_copy(tb, tabs, T_ROW * 2);
-  load_w(wbf + woff, nullptr, wt);
+  load_wt(wbf + woff, wt);
   pdl_wait();
   float gw[2][4][4];  // grad W [16 o][8 i] tiles of this warp's pixels
   float2 gb[2][2];    // sums of dpre over the thread's even and odd pixels, channels 16 m + 8 e + g
@@ -1384,7 +1354,7 @@ __global__ void __launch_bounds__(NTH, 2) fno_lift_bwd(const float* __restrict__
     load_inputs(u_in, f, fps, b, iy0, us, fs);
     cp_wait_all();
     __syncthreads();
-    row_inverse(zs, tb, gs, true);
+    row_inverse(zs, tb, gs);
     features(us, fs, iy0, as);
     __syncthreads();
     {  // grad W0 += dv0 a^T: M = FC, N = 8, K = NP split over warp quarters

@@ -84,13 +84,14 @@ constexpr int WS_NB = 192;  // most accumulator columns of the warp-specialised 
 //          out0 = partials [(ks T + t) M + m].
 // ADJ = 1: A = Ht [rows = Nf][lda = 2 M], all of K = 2 M, small operand from w [T][M];
 //          out0 = z [t Nf + n], out1 (may be null) = conj(f) z.
-// NB = 2T rounded up to one of 32, 64, 96, 128, 192, 256 accumulator columns.  Each chunk's 12 MMAs start a
+// For more than 96 and up to 128 transmitters: NB = 256 accumulator columns.  Each chunk's 12 MMAs start a
 // fresh accumulator, alternating between two TMEM buffers: while chunk c's MMAs run, the threads add chunk
 // c - 1's result into FP32 registers (round to nearest).  The tensor cores' FP32 accumulation rounds its sums
 // more coarsely: accumulating a whole split in TMEM (64 to 432 chunks, hundreds of MMAs) left the products
 // 1.2e-5 to 1.5e-5 from FP64 on random inputs; with chains of 12 they are within 8e-7 (C2, C3 sizes).
-template <int ADJ, int NB>
-__global__ void __launch_bounds__(STH, NB > 128 ? 1 : 2) sense_tc_kernel(const float* __restrict__ A, long long lda, long long rows,
+constexpr int TC_NB = 256, TC_SMEM = 2 * SPA + 2 * (TC_NB / 8) * SSBO;
+template <int ADJ>
+__global__ void __launch_bounds__(STH, 1) sense_tc_kernel(const float* __restrict__ A, long long lda, long long rows,
                                                        long long K, long long KS, const float2* __restrict__ src,
                                                        long long lds, const float2* __restrict__ f, long long NP,
                                                        int T, int M, long long Nf, float2* __restrict__ out0,
@@ -98,9 +99,9 @@ __global__ void __launch_bounds__(STH, NB > 128 ? 1 : 2) sense_tc_kernel(const f
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tslot;
-  constexpr int SPB = (NB / 8) * SSBO;
+  constexpr int NB = TC_NB, SPB = (NB / 8) * SSBO;
   constexpr int NH = NB / 2;  // accumulator columns per thread
-  constexpr uint32_t ncol = 2 * NB <= 64 ? 64u : 2 * NB <= 128 ? 128u : 2 * NB <= 256 ? 256u : 512u;
+  constexpr uint32_t ncol = 2 * NB;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long row0 = (long long)blockIdx.x * 128;
   const long long kb = ADJ ? 0 : (long long)blockIdx.y * KS;
@@ -651,13 +652,12 @@ cisor_status sense_tc_setup(cisor_ctx* c) {
       CISOR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ws_smem(nb)));
     return CISOR_OK;
   }
-  const int smem = 2 * SPA + 2 * (nb / 8) * SSBO;
-  for (const void* fn : {(const void*)sense_tc_kernel<0, 256>, (const void*)sense_tc_kernel<1, 256>}) {
-    CISOR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  for (const void* fn : {(const void*)sense_tc_kernel<0>, (const void*)sense_tc_kernel<1>}) {
+    CISOR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
     CISOR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   }
   int occ = 0;
-  CISOR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sense_tc_kernel<0, 256>, STH, smem));
+  CISOR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sense_tc_kernel<0>, STH, TC_SMEM));
   c->sense_tc_occ = occ < 1 ? 1 : occ;
   return CISOR_OK;
 }
@@ -723,7 +723,7 @@ static cisor_status sense_tc_gemm(cisor_ctx* c, long long rows, long long K, lon
         A, rows, rtiles, nitems, K, KS, src, lds, f, c->N, ntx, c->M, c->Nf,
         out0, out1, c->tc_err);
   } else {
-    sense_tc_kernel<ADJ, 256><<<dim3((unsigned)rtiles, (unsigned)splits), STH, 2 * SPA + 2 * 32 * SSBO, c->stream>>>(
+    sense_tc_kernel<ADJ><<<dim3((unsigned)rtiles, (unsigned)splits), STH, TC_SMEM, c->stream>>>(
         A, K, rows, K, KS, src, lds, f, c->N, ntx, c->M, c->Nf, out0,
         out1, c->tc_err);
   }

@@ -33,30 +33,20 @@
 
 namespace cisor {
 
-// Dual planes: component k of plane c at (dim * c + k) * N.
+// z as planes and, for the 3D iterations, r = p = 0 (r null: none follow).  Dual planes: component k of plane c at
+// (3 c + k) * N.
 __global__ void tv_split_kernel(const float2* __restrict__ z, float* __restrict__ zp, float* __restrict__ r,
-                                float* __restrict__ p, long long N, int ncomp, int dim) {
+                                float* __restrict__ p, long long N, int ncomp) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   const float2 v = z[i];
   zp[i] = v.x;
   if (ncomp == 2) zp[N + i] = v.y;
-  for (int k = 0; k < dim * ncomp; ++k) {
+  if (!r) return;
+  for (int k = 0; k < 3 * ncomp; ++k) {
     r[k * N + i] = 0.f;
     p[k * N + i] = 0.f;
   }
-}
-
-// (D^T r)(iy, ix) for the forward difference with zero difference at the last index
-__device__ __forceinline__ float dt_at(const float* __restrict__ rx, const float* __restrict__ ry, int iy, int ix,
-                                       int n) {
-  const int i = iy * n + ix;
-  float v = 0.f;
-  if (ix < n - 1) v -= rx[i];
-  if (ix > 0) v += rx[i - 1];
-  if (iy < n - 1) v -= ry[i];
-  if (iy > 0) v += ry[i - n];
-  return v;
 }
 
 // Several FGP iterations of a 2D image per launch.  A CTA loads a TVR x TVR region of z, r and p, one pixel a
@@ -66,7 +56,7 @@ __device__ __forceinline__ float dt_at(const float* __restrict__ rx, const float
 // both compute.  Pixels outside the image hold r = 0, which is what the differences' boundary terms need (r is also
 // 0 at the last index of its own direction, where the difference is zero).
 // One launch per iteration spent 5 us on launch and memory latency for 1 us of arithmetic: 20 iterations of a
-// complex 256 x 256 image took 115 us as a call and now take 48 us (real 64 x 64: 99 -> 30 us).  What is left is
+// complex 256 x 256 image took 118 us as a call and now take 45 us (real 64 x 64: 99 -> 30 us).  What is left is
 // the latency of the iterations themselves (two barriers, a square root and two divisions, 0.4 us each).  More
 // iterations a launch (7, 10) recompute more halo than the launches cost at 256 x 256 (61 and 115 us); wider
 // regions with several pixels a thread (48 x 48, 64 x 64) leave too few threads to hide the divisions (64 to 84 us).
@@ -204,7 +194,7 @@ static cisor_status tv_blocks(cisor_ctx* c, const float2* z, float2* x, double l
   return CISOR_OK;
 }
 
-// (D^T r) at voxel (iz, iy, ix) of an n^3 volume
+// (D^T r) at voxel (iz, iy, ix) of an n^3 volume, for the forward difference with zero difference at the last index
 __device__ __forceinline__ float dt3_at(const float* __restrict__ rx, const float* __restrict__ ry,
                                         const float* __restrict__ rz, int iz, int iy, int ix, int n) {
   const long long nn = (long long)n * n;
@@ -259,19 +249,18 @@ __global__ void tv_iter3_kernel(const float* __restrict__ zp, const float* __res
   ro[2 * N + i] = pz + beta * (pz - poz);
 }
 
-__global__ void tv_final_kernel(const float* __restrict__ zp, const float* __restrict__ p, int n, int dim, float lam,
+// x = P_C(z - lam D^T p) of a volume, or the clamp of N values where lam = 0, and the momentum
+__global__ void tv_final_kernel(const float* __restrict__ zp, const float* __restrict__ p, int n, long long N, float lam,
                                 float lo0, float hi0, float lo1, float hi1, int ncomp, float2* x, const float2* fprev,
                                 float beta_mom, float2* __restrict__ s_out) {
-  const long long N = dim == 3 ? (long long)n * n * n : (long long)n * n;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   const int ix = (int)(i % n), iy = (int)((i / n) % n), iz = (int)(i / ((long long)n * n));
   float xv[2] = {0.f, 0.f};
   for (int c = 0; c < ncomp; ++c) {
     const float lo = c ? lo1 : lo0, hi = c ? hi1 : hi0;
-    const float* pc = p + dim * c * N;
-    float d = 0.f;
-    if (lam > 0.f) d = dim == 3 ? dt3_at(pc, pc + N, pc + 2 * N, iz, iy, ix, n) : dt_at(pc, pc + N, iy, ix, n);
+    const float* pc = p + 3 * c * N;
+    const float d = lam > 0.f ? dt3_at(pc, pc + N, pc + 2 * N, iz, iy, ix, n) : 0.f;
     xv[c] = fminf(fmaxf(zp[c * N + i] - lam * d, lo), hi);
   }
   const float2 xo = make_float2(xv[0], xv[1]);
@@ -390,19 +379,19 @@ cisor_status tv_prox(cisor_ctx* c, const float2* z, float2* x, double lam, int i
   const long long N = c->N;
   const int ncomp = complex_f ? 2 : 1;
   const unsigned gN = (unsigned)((N + 255) / 256);
-  const int dim = c->dim;
-  if (dim == 2 && lam > 0.0 && iters > 0)
+  const bool tv = lam > 0.0 && iters > 0;  // else the clamp
+  if (c->dim == 2 && tv)
     return tv_blocks(c, z, x, lam, iters, lo, hi, lo_im, hi_im, ncomp, f_prev, beta_mom, s_out);
-  tv_split_kernel<<<gN, 256, 0, c->stream>>>(z, c->tv_z, c->tv_r0, c->tv_p, N, ncomp, dim);
+  tv_split_kernel<<<gN, 256, 0, c->stream>>>(z, c->tv_z, tv ? c->tv_r0 : nullptr, c->tv_p, N, ncomp);
   CISOR_CUDA(cudaGetLastError());
   c->launches += 1;
-  if (dim == 3 && lam > 0.0 && iters > 0) {
+  if (tv) {
     const int bx = ((n + 31) / 32) * 32 > 256 ? 256 : ((n + 31) / 32) * 32;
     dim3 g((n + bx - 1) / bx, n, n * ncomp);
     double t = 1.0;
     float* rin = c->tv_r0;
     float* rout = c->tv_r1;
-    const float step = (float)(1.0 / (4.0 * dim * lam));
+    const float step = (float)(1.0 / (12.0 * lam));
     for (int k = 0; k < iters; ++k) {
       const double tn = (1.0 + sqrt(1.0 + 4.0 * t * t)) / 2.0;
       const float beta = (float)((t - 1.0) / tn);
@@ -416,8 +405,7 @@ cisor_status tv_prox(cisor_ctx* c, const float2* z, float2* x, double lam, int i
       t = tn;
     }
   }
-  const float lam_f = (lam > 0.0 && iters > 0) ? (float)lam : 0.f;
-  tv_final_kernel<<<gN, 256, 0, c->stream>>>(c->tv_z, c->tv_p, n, dim, lam_f, (float)lo, (float)hi, (float)lo_im,
+  tv_final_kernel<<<gN, 256, 0, c->stream>>>(c->tv_z, c->tv_p, n, N, tv ? (float)lam : 0.f, (float)lo, (float)hi, (float)lo_im,
                                              (float)hi_im, ncomp, x, f_prev, (float)beta_mom, s_out);
   CISOR_CUDA(cudaGetLastError());
   c->launches += 1;

@@ -13,9 +13,10 @@
 // the grid count as zero).  The forward matvec runs the stencil as the
 // epilogue of the convolution (A x, b - A x and the dot slots of the Krylov
 // solver); the adjoint runs it before the convolution, whose inverse-row
-// epilogue then forms the result.  Dot partials of both land in
-// [T][3 nblk][DOT_SLOTS] (component-major), the layout the solver's scalar
-// step sums.
+// epilogue then forms the result.  Dot partials of both land in the
+// [T][3 nblk][DOT_SLOTS] slots that the solver's scalar step sums: the adjoint's
+// as nblk per component, the forward's one per CTA over all components with
+// zeros in the slots behind them.
 //
 // Tables: H~ [M, 3N] = delta^3 times row 3 of the dyadic Green's function
 //     G(r) = k^2 [ (3/(kd)^2 - 3j/(kd) - 1) r^ r^T + (1 + j/(kd) - 1/(kd)^2) I ] g(d)
@@ -103,7 +104,7 @@ __global__ void __launch_bounds__(256, 3) vec_stencil_kernel(const VecEpiArgs a)
     float2 n0, n1, nd0, nd1;
     load(z0 - 1, m0[0], m1[0], m2[0], c2[0], n0, n1, nd0, nd1);
     load(z0, m0[1], m1[1], m2[1], c2[1], c0, c1, d0, d1);
-constexpr int UN = DK > DOTS_NONE ? 1 : 2;  // (inner products leave no registers for two planes)
+    constexpr int UN = DK > DOTS_NONE ? 1 : 2;  // (inner products leave no registers for two planes)
 #pragma unroll UN
     for (int z = z0; z < z1; ++z) {
       const long long i0 = base + (long long)z * n2 + col;
