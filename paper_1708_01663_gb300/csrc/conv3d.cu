@@ -14,12 +14,13 @@
 // padded intermediate through HBM five times, growing it to n P^2 values
 // between the y and z kernels: 2.4 GB a pass at 48 transforms of n = 64, P =
 // 128.  Here it never leaves n^2 P values and moves twice (0.8 GB); a plane's
-// 64 KB fit one SM's shared memory with room for two CTAs.  Measured, one pass:
+// 64 KB and the 32 KB of its column exchanges leave room for two CTAs an SM.  Measured, one pass:
 // 48 transforms of n = 64 554 -> 465 us (two-stage column kernels before), 243
 // of n = 32 (81 vectorial fields, with their stencil) 400 -> 305 us, 20 of n = 40
-// 223 -> 130 us; no size measured is slower.  The plane kernel (80 % of the pass)
-// is bound by shared-memory traffic (its pipe 72 % busy, issue 60 %): the two
-// exchanges and the passes over the plane between the directions.
+// 223 -> 130 us; no size measured is slower.  The plane kernel (69 %
+// of a pass of eight transforms of n = 64) is bound by shared-memory traffic (its
+// pipe 72 % busy, issue 60 %, FMA pipe 45 %, DRAM 8 %): the two exchanges and the
+// passes over the plane between the directions.
 //
 // Transforms are two-stage, P = E x 8 (128 = 16 x 8, 64 = 8 x 8): E elements a
 // thread, 8 threads a transform, one exchange each way, arranged as

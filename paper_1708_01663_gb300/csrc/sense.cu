@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(256, 2) sense_fwd_kernel(const float2* __restr
 // D += 1/2 sum |w|^2.  A CTA takes 32 consecutive entries (lanes, coalesced); its 8 warps sum the partials
 // k = w, w + 8, ... and warp 0 adds the 8 sums in warp order (the same order every call).  All of it in three FP32
 // values a sum and one conversion an entry (fp32_sum.cuh: no less exact than FP64, which runs at a small fraction of
-// the FP32 rate: 256 splits of 48 x 1024 entries 671 -> 593 us for the product, 147 of 64 x 256 76 -> 67, this kernel
+// the FP32 rate: 256 splits of 48 x 1024 entries 671 -> 593 us for the product, 76 of 64 x 256 76 -> 67, this kernel
 // 15 -> 7 us there).  A sum that is not finite is taken again in FP64, whose range is wider.  Four partials a step: eight
 // or two are 0.5 to 1 us slower where a warp has six.
 constexpr int RED_WARPS = 8;

@@ -23,9 +23,9 @@
 //
 // Up to 96 transmitters (NB <= 192) H and Ht are stored as those tiles: 128 rows
 // by 32 floats, contiguous, in the order in which a CTA streams them (tile_off), so
-// that a chunk is one 16 KB bulk copy by one thread; the copies alone run at 7.3
-// TB/s.  One warp-specialised CTA per SM runs over the tiles (sense_ws_kernel): a
-// thread keeps SENSE_STAGES bulk copies of the big operand in flight, converter
+// that a chunk is one 16 KB bulk copy by one thread (sense_tile.cuh); the copies
+// alone, which only read, run at 7.3 TB/s (a copy that also writes moves 6.8).  One
+// warp-specialised CTA per SM runs over the tiles (sense_ws_kernel): a thread keeps SENSE_STAGES bulk copies of the big operand in flight, converter
 // warps split each chunk into hi / lo planes in TENSOR MEMORY, builder warps write
 // the small operand's planes to shared memory, two threads issue the MMAs (A from
 // tensor memory, B from shared memory) and the remaining warps add finished chunks
@@ -38,10 +38,10 @@
 // 1.15 -> 0.60 ms, adjoint 0.93 -> 0.58 ms against the kernel below on row-major
 // matrices, which does all roles in every thread; 64 transmitters, 256 receivers,
 // 256^2: 0.136 -> 0.071, 0.092 -> 0.082; 81, 36, 32^3 vectorial: 0.108 -> 0.095,
-// 0.096 -> 0.068; 8, 360, 128^2: 0.044 -> 0.024, 0.037 -> 0.017; 8, 32, 64^2: 0.017 -> 0.015,
-// 0.008 -> 0.007 (all launches; slower only with two receivers and many
-// transmitters, whose chunks are mostly padding: 48, 2, 256^2 adjoint 20 -> 24
-// us).  What bounds it: the hand-overs between the roles (below); the MMAs keep
+// 0.096 -> 0.065; 8, 360, 128^2: 0.044 -> 0.022, 0.037 -> 0.017; 8, 32, 64^2: 0.017 -> 0.014,
+// 0.008 -> 0.007 (all launches; slower only with a few receivers and many
+// transmitters, whose chunk is computed whole however narrow it is: 48, 2, 256^2
+// adjoint 20 -> 23 us).  What bounds it: the hand-overs between the roles (below); the MMAs keep
 // the tensor pipe about half of the time at NB = 96, the copies the memory for
 // half.  More than 96 transmitters leave no room for two
 // accumulators and A in tensor memory and take the kernel below (sense_tc_kernel).
@@ -57,9 +57,11 @@ constexpr int SLBO = 144, SSBO = 8 * SLBO;   // K-group and 8-row strides of the
 constexpr int SPA = 16 * SSBO;               // bytes of one plane of the 128-row tile
 constexpr int STH = 256;                     // threads per CTA
 constexpr int S_WAIT = 1 << 20;              // polls of the MMA completion barrier before giving up
-// K (floats) per CTA of the forward GEMM: splits of 64 chunks, 2048 and more CTAs at C3, measured faster than one
-// wave of 432-chunk CTAs (1.04 against 1.59 ms): CTAs that start together read the same slab of the small
-// operand, which then stays in L2 while H streams past it.
+// K (floats) per split of the forward GEMM, at most.  sense_tc_kernel, a CTA per split and row tile: splits of 64 chunks,
+// 2048 and more CTAs at 48 transmitters, 1024 receivers, 64^3, measured faster than one wave of 432-chunk CTAs (1.04
+// against 1.59 ms): CTAs that start together read the same slab of the small operand, which then stays in L2 while H
+// streams past it.  sense_ws_kernel, whose persistent CTAs take splits as items, in the same order: 16, 32 and 64 chunks
+// 594 us there, 128 564, 256 628; 64, 256, 256^2 87, 78, 67, 67, 67.
 constexpr long long S_KMAX = 64 * SK;
 constexpr long long S_MAX = 256;  // at most this many splits (partials T x M x 8 bytes each)
 
