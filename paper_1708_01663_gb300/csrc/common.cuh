@@ -230,6 +230,7 @@ struct ConvOp {
                           // model run as consecutive transforms; 0 or 1: one)
   int tx0;                // first transform of this launch (set by conv_pass when it splits a pass
                           // into transmitter chunks; R is indexed from the chunk's start)
+  int pass_ntx;           // transforms of the whole pass (likewise)
 };
 enum { PRO_COPY = 0, PRO_PUPDATE = 1, PRO_AXPY = 2 };
 // Programmatic dependent launch (sm_90 and later): the solver chain's kernels

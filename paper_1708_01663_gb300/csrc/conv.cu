@@ -543,7 +543,8 @@ static void launch_cols_2s(cisor_ctx* c, const ConvOp& op, int nslab, long long 
 // transform outside an iteration keeps the two-stage kernel: 11.8 against 13.1 us a pass at 256^2, equal at 129^2.
 template <int P>
 static int cols_shape(const cisor_ctx* c, const ConvOp& op) {
-  if (P != 512 || !c->cols_auto || op.ntx >= 6 || (op.ntx == 1 && !op.active)) return c->cols_nt;
+  const int nt = op.pass_ntx;  // of the whole pass: its chunks take the same kernel, so that results do not depend on them
+  if (P != 512 || !c->cols_auto || nt >= 6 || (nt == 1 && !op.active)) return c->cols_nt;
   return 512;
 }
 
@@ -646,6 +647,7 @@ static cisor_status conv_pass_t(cisor_ctx* c, const ConvOp& op) {
   const int chunk = (c->tx_chunk > 0 && c->tx_chunk < op.ntx) ? c->tx_chunk : op.ntx;
   for (int t0 = 0; t0 < op.ntx; t0 += chunk) {
     ConvOp o = op;
+    o.pass_ntx = op.ntx;
     o.tx0 = op.tx0 + t0;
     o.ntx = op.ntx - t0 < chunk ? op.ntx - t0 : chunk;
     CISOR_TRY(conv_chunk_t<P>(c, o));

@@ -61,3 +61,21 @@ def test_few_transforms_p512(T):
     assert np.array_equal(A[None], A[same]) and not np.array_equal(A[None], A[other])
     for shape in (512, 16):
         assert rel(u[None], u[shape]) < 1e-5
+
+
+@pytest.mark.parametrize("T,chunk", [(5, 2), (7, 3), (7, 1)])
+def test_chunks_keep_the_shape_p512(T, chunk):
+    """Transmitter chunks take the kernel of the whole pass: identical results, as for shapes that were set."""
+    build.build()
+    n = 129
+    ctx = cisor.Cisor(n, 0.125, synth.plane_wave_angles(T), synth.circle_receivers(8, 0.125 * n), complex_f=True)
+    f = c64(synth.ellipse_phantom(n, 3, (0.05, 0.2), 31, 0.02))
+    x = c64(synth.random_field(9, (T, n, n)))
+    y, u = [], []
+    for k in (0, chunk):
+        ctx.set_tx_chunk(k)
+        y.append(np.empty_like(x))
+        u.append(np.empty_like(x))
+        ctx.apply_A(f, x, y[-1])
+        ctx.forward(f, u_out=u[-1], tol=1e-6, max_iter=2000)
+    assert np.array_equal(y[0], y[1]) and np.array_equal(u[0], u[1])
