@@ -133,7 +133,8 @@ cisor_status cisor_sizes(const cisor_ctx* ctx, int* n, int* P, int* T, int* M, l
  * of G (Eq. 3 through Sec. III-A's FFT convolution): [P, P] complex64. */
 cisor_status cisor_green_spectrum(cisor_ctx* ctx, void* ghat_out);
 
-/* Copy out H (Eq. 2): [M, N] complex64. */
+/* Copy out H (Eq. 2): [M, N] complex64.  The first copy to host memory may
+ * allocate device buffers of up to 64 MB, which the context keeps. */
 cisor_status cisor_sensing_matrix(cisor_ctx* ctx, void* H_out);
 
 /* Copy out the incident fields u_in: [T, N] complex64. */
@@ -298,7 +299,9 @@ cisor_status cisor_set_tx_chunk(cisor_ctx* ctx, int tx_chunk);
 cisor_status cisor_set_solve_loop(cisor_ctx* ctx, int device_loop);
 
 /* The context's current column shape (512, 256 or 16) and transmitter chunk
- * (0 = none); either output may be NULL. */
+ * (0 = none); either output may be NULL.  Until the shape is set or autotuned
+ * it is a default by size, and at P = 512 a pass of two to five transforms
+ * takes 512 whatever it says. */
 cisor_status cisor_tuning(const cisor_ctx* ctx, int* cols_nt, int* tx_chunk);
 
 /* Per-transmitter receiver mask (the Fresnel set-ups of Sec. IV record each
