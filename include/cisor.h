@@ -300,8 +300,8 @@ cisor_status cisor_set_solve_loop(cisor_ctx* ctx, int device_loop);
 
 /* The context's current column shape (512, 256 or 16) and transmitter chunk
  * (0 = none); either output may be NULL.  Until the shape is set or autotuned
- * it is a default by size, and at P = 512 a pass of two to five transforms
- * takes 512 whatever it says. */
+ * it is a default by size, and at P = 512 the iterations of solves for one
+ * or three to five transmitters run 512 threads whatever it says. */
 cisor_status cisor_tuning(const cisor_ctx* ctx, int* cols_nt, int* tx_chunk);
 
 /* Per-transmitter receiver mask (the Fresnel set-ups of Sec. IV record each

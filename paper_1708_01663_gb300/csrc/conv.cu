@@ -168,7 +168,7 @@ template <int P, int MODE, int NT> struct ColSmem {
 };
 
 // D3 = false (2D) fixes es = P and a single slab at compile time.
-template <int P, int MODE, bool ADJ, int NT, bool D3>
+template <int P, int MODE, bool ADJ, int NT, bool D3, bool TWALL = ColSmem<P, MODE, NT>::TWALL>
 __global__ void __launch_bounds__(NT, 1024 / NT) conv_cols(const int* __restrict__ active, const float2* __restrict__ tw_g,
                                                     const float2* __restrict__ ghat, float2* __restrict__ R,
                                                     const ColGeo geo) {
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) conv_cols(const int* __restrict
         const int i = PL::elem(lt, q, r, R0);
         v[q * R0 + r] = (PL::lower(q, r, R0) && i < n) ? base[i * es] : make_float2(0.f, 0.f);
       }
-    reg_fft<P, false, false, true, SM::TWALL, SM::PING>(v, buf, lay, lay, lt, tw, CtaSync(), buf2);
+    reg_fft<P, false, false, true, TWALL, SM::PING>(v, buf, lay, lay, lt, tw, CtaSync(), buf2);
   }
   constexpr int RL = PL::template last<false>();
   if (MODE == COL_FWD) {
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) conv_cols(const int* __restrict
   }
   // PING: both transforms use buf, then buf2, and each exchange's barrier orders the reads of
   // the one before (reg_fft); otherwise the leading barrier of each exchange does
-  reg_fft<P, true, true, false, SM::TWALL, SM::PING>(v, buf, layr, layr, lt, twr, CtaSync(), buf2);
+  reg_fft<P, true, true, false, TWALL, SM::PING>(v, buf, layr, layr, lt, twr, CtaSync(), buf2);
   constexpr int RI = PL::template last<true>();
 #pragma unroll
   for (int q = 0; q < 8 / RI; ++q)
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(256) conv_rows_inv(const ConvOp op, const floa
     block_dots<256, DotSlots<DK>::MASK>(acc, reinterpret_cast<float2*>(op.part) + ((size_t)tx * nblk + blockIdx.x) * DOT_SLOTS);
 }
 
-template <int P, int MODE, bool ADJ, int NT>
+template <int P, int MODE, bool ADJ, int NT, bool TWALL = ColSmem<P, MODE, NT>::TWALL>
 static void launch_cols(cisor_ctx* c, const ConvOp& op, int nslab, long long es, long long slab) {
   constexpr int W = ConvCfg<P>::template Col<NT>::W;
   constexpr size_t SMB = ColSmem<P, MODE, NT>::BYTES;
@@ -469,20 +469,22 @@ static void launch_cols(cisor_ctx* c, const ConvOp& op, int nslab, long long es,
     }
   }
   if constexpr (MODE == COL_G)
-    (void)launch_pdl(conv_cols<P, MODE, ADJ, NT, false>, g, dim3(NT), SMB, c->stream, op.active, c->twst, c->ghat, c->R,
-                     geo);
+    (void)launch_pdl(conv_cols<P, MODE, ADJ, NT, false, TWALL>, g, dim3(NT), SMB, c->stream, op.active, c->twst, c->ghat,
+                     c->R, geo);
 }
 
 // The column kernels' dynamic shared memory may exceed the 48 KB default: raise
 // each instantiation's limit once, when a context picks its FFT size.
-template <int P, int MODE, bool ADJ, int NT, bool D3>
+template <int P, int MODE, bool ADJ, int NT, bool D3, bool TWALL = ColSmem<P, MODE, NT>::TWALL>
 static cudaError_t cols_attr() {
-  return cudaFuncSetAttribute(conv_cols<P, MODE, ADJ, NT, D3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(conv_cols<P, MODE, ADJ, NT, D3, TWALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)ColSmem<P, MODE, NT>::BYTES);
 }
 template <int P, bool ADJ, int NT>
 static cudaError_t cols_attrs() {
   cudaError_t e = cols_attr<P, COL_G, ADJ, NT, false>();
+  if constexpr (P == 512 && NT == 512)
+    if (e == cudaSuccess) e = cols_attr<P, COL_G, ADJ, NT, false, true>();
   if constexpr (P == 256) {
     if (e == cudaSuccess) e = cols_attr<P, COL_G, ADJ, NT, true>();
     if (e == cudaSuccess) e = cols_attr<P, COL_FWD, ADJ, NT, true>();
@@ -535,17 +537,19 @@ static void launch_cols_2s(cisor_ctx* c, const ConvOp& op, int nslab, long long 
   }
 }
 
-// The column shape of one pass: the context's.  Until that is set or autotuned, fewer than six transforms at P = 512
-// take 512 threads instead of the two-stage kernel, whose 32 CTAs a transform leave most SMs idle while each works
-// longer: an iteration of a solve takes 41.1, 49.3 and 49.2 us with one, four and five transmitters at 129^2 against
-// 45.2, 53.0 and 52.9, at 256^2 41.6, 54.1, 57.2 against 46.0, 55.8, 59.6 (two transmitters within 3 % either way; six
-// are faster with the two-stage kernel, 61.8 against 64.1, seven vary by size, eight 65.1 against 71).  A single
-// transform outside an iteration keeps the two-stage kernel: 11.8 against 13.1 us a pass at 256^2, equal at 129^2.
+// The column shape of one pass: the context's.  Until that is set or autotuned, the iterations of a solve with fewer
+// than six transforms at P = 512 take 512 threads, with all twiddles from the table, instead of the two-stage kernel,
+// whose 32 CTAs a transform leave most SMs idle while each works longer.  An iteration takes 42.4, 46.5, 49.4 and 49.8
+// us with one, three, four and five transmitters at 129^2 against 45.5, 50.0, 54.0 and 53.1, at 256^2 42.1, 51.2, 54.8
+// and 56.8 against 45.6, 52.1, 55.9 and 59.2.  Two and six keep the two-stage kernel (45.2 against 46.0 and 53.8 against
+// 54.4 at 129^2, 50.1 as well and 61.5 against 64.1 at 256^2).  G f x is 2.5e-7 from FP64 at 129^2, 2.7e-7 with the two-stage kernel and 3.0e-7 with 512 threads that
+// form the twiddles as products (faster with many transforms only).  Passes outside an iteration gain nothing.
+constexpr int COLS_TABLE = 513;  // (not a shape to be set)
 template <int P>
 static int cols_shape(const cisor_ctx* c, const ConvOp& op) {
-  const int nt = op.pass_ntx;  // of the whole pass: its chunks take the same kernel, so that results do not depend on them
-  if (P != 512 || !c->cols_auto || nt >= 6 || (nt == 1 && !op.active)) return c->cols_nt;
-  return 512;
+  // the transforms of the whole pass: its chunks take the same kernel, so that results do not depend on them
+  const int nt = op.pass_ntx;
+  return P == 512 && c->cols_auto && op.active && nt < 6 && nt != 2 ? COLS_TABLE : c->cols_nt;
 }
 
 template <int P, int MODE>
@@ -558,6 +562,14 @@ static void cols_pass(cisor_ctx* c, const ConvOp& op, int nslab, long long es, l
       launch_cols_2s<P, MODE, false>(c, op, nslab, es, slab);
     return;
   }
+  if constexpr (P == 512)
+    if (shape == COLS_TABLE) {
+      if (op.adjoint)
+        launch_cols<P, MODE, true, 512, true>(c, op, nslab, es, slab);
+      else
+        launch_cols<P, MODE, false, 512, true>(c, op, nslab, es, slab);
+      return;
+    }
   if (shape == 256) {
     if (op.adjoint)
       launch_cols<P, MODE, true, 256>(c, op, nslab, es, slab);

@@ -41,26 +41,28 @@ def test_columns_3d_p256(n, shape):
 
 @pytest.mark.parametrize("T", [1, 2, 5, 6])
 def test_few_transforms_p512(T):
-    """By default a pass has the bits of 512 threads for two to five transforms, of the two-stage columns otherwise; solves,
-    which mix them with one transmitter, agree with both shapes (1e-5, as solves to 1e-6 by different shapes do)."""
+    """By default a pass has the bits of the two-stage columns; solves of one and of three to five transmitters iterate with
+    another kernel and agree with both shapes that can be set (1e-5, as solves to 1e-6 by different shapes do)."""
     build.build()
     n = 129
     new = lambda: cisor.Cisor(n, 0.125, synth.plane_wave_angles(T), synth.circle_receivers(8, 0.125 * n), complex_f=True)
     f = c64(synth.ellipse_phantom(n, 3, (0.05, 0.2), 31, 0.02))
     x = c64(synth.random_field(9, (T, n, n)))
-    A, u = {}, {}
+    A, u, g = {}, {}, {}
+    y = c64(synth.random_field(10, (T, 8)))
     for shape in (None, 512, 16):
         ctx = new()
         if shape:
             ctx.set_cols_cta(shape)
-        A[shape], u[shape] = np.empty_like(x), np.empty_like(x)
+        A[shape], u[shape], g[shape] = np.empty_like(x), np.empty_like(x), np.empty_like(f)
         ctx.apply_A(f, x, A[shape])
         ctx.forward(f, u_out=u[shape], tol=1e-6, max_iter=2000)
+        ctx.grad(f, y, g[shape], tol=1e-6, max_iter=2000)
         ctx.close()
-    same, other = (512, 16) if 2 <= T < 6 else (16, 512)
-    assert np.array_equal(A[None], A[same]) and not np.array_equal(A[None], A[other])
+    assert np.array_equal(A[None], A[16])
+    assert np.array_equal(u[None], u[16]) == (T not in (1, 5))
     for shape in (512, 16):
-        assert rel(u[None], u[shape]) < 1e-5
+        assert rel(u[None], u[shape]) < 1e-5 and rel(g[None], g[shape]) < 1e-5
 
 
 @pytest.mark.parametrize("T,chunk", [(5, 2), (7, 3), (7, 1)])
