@@ -21,6 +21,11 @@ struct Fp32Sum {
     return r;
   }
   CISOR_SUM_HD void add(float p) { c += two_sum(e, two_sum(s, p)); }
+  CISOR_SUM_HD void add(const Fp32Sum& o) {
+    add(o.s);
+    c += two_sum(e, o.e);
+    c += o.c;
+  }
   CISOR_SUM_HD double value() const { return (double)s + ((double)e + (double)c); }
 };
 

@@ -118,10 +118,12 @@ __global__ void __launch_bounds__(256, 2) sense_fwd_kernel(const float2* __restr
 // D += 1/2 sum |w|^2.  A CTA takes 32 consecutive entries (lanes, coalesced); its 8 warps sum the partials
 // k = w, w + 8, ... and warp 0 adds the 8 sums in warp order (the same order every call).  All of it in three FP32
 // values a sum and one conversion an entry (fp32_sum.cuh: no less exact than FP64, which runs at a small fraction of
-// the FP32 rate: 256 splits of 48 x 1024 entries 671 -> 593 us for the product, 76 of 64 x 256 76 -> 67, this kernel
-// 15 -> 7 us there).  A sum that is not finite is taken again in FP64, whose range is wider.  Four partials a step: eight
-// or two are 0.5 to 1 us slower where a warp has six.
-constexpr int RED_WARPS = 8;
+// the FP32 rate: 256 splits of 48 x 1024 entries 671 -> 593 us for the product, 76 of 64 x 256 76 -> 67).  A sum that is
+// not finite is taken again in FP64, whose range is wider.  Otherwise bound by the latency of the partials, so a warp
+// asks for RED_LOADS at a time, the last ones guarded: this kernel takes 5.8, 4.2, 4.5 and 6.7 us for 48 x 2, 8 x 32, 8 x
+// 360 and 64 x 256 entries of 147, 64, 49 and 76 splits, with four loads unrolled and a loop over the rest 8.9, 5.4, 6.0
+// and 7.0, in FP64 10.1, 8.7, 6.3 and 14.8.
+constexpr int RED_WARPS = 8, RED_LOADS = 8;
 __global__ void __launch_bounds__(32 * RED_WARPS) sense_reduce_kernel(const float2* __restrict__ part, int ks, int T,
                                                                      int M, const float2* __restrict__ y,
                                                                      float2* __restrict__ Z, float2* __restrict__ w,
@@ -133,11 +135,19 @@ __global__ void __launch_bounds__(32 * RED_WARPS) sense_reduce_kernel(const floa
   const long long TM = (long long)T * M;
   Fp32Sum a, b;  // real and imaginary parts
   if (idx < TM) {
-#pragma unroll 4
-    for (int k = warp; k < ks; k += RED_WARPS) {
-      const float2 p = part[(long long)k * TM + idx];
-      a.add(p.x);
-      b.add(p.y);
+    for (int k0 = warp; k0 < ks; k0 += RED_LOADS * RED_WARPS) {  // loads together, also where fewer are left
+      float2 p[RED_LOADS];
+#pragma unroll
+      for (int j = 0; j < RED_LOADS; ++j) {
+        const int k = k0 + j * RED_WARPS;
+        if (k < ks) p[j] = part[(long long)k * TM + idx];
+      }
+#pragma unroll
+      for (int j = 0; j < RED_LOADS; ++j) {
+        if (k0 + j * RED_WARPS >= ks) break;
+        a.add(p[j].x);
+        b.add(p[j].y);
+      }
     }
   }
   const float own[6] = {a.s, a.e, a.c, b.s, b.e, b.c};
@@ -148,12 +158,10 @@ __global__ void __launch_bounds__(32 * RED_WARPS) sense_reduce_kernel(const floa
   double d = 0.0;
   if (idx < TM) {
 #pragma unroll
-    for (int i = 1; i < RED_WARPS; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        a.add(red[i][j][lane]);
-        b.add(red[i][3 + j][lane]);
-      }
+    for (int i = 1; i < RED_WARPS; ++i) {
+      a.add(Fp32Sum{red[i][0][lane], red[i][1][lane], red[i][2][lane]});
+      b.add(Fp32Sum{red[i][3][lane], red[i][4][lane], red[i][5][lane]});
+    }
     double sx = a.value(), sy = b.value();
     if (!isfinite(sx) || !isfinite(sy)) {
       sx = sy = 0.0;

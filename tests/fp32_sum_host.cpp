@@ -33,15 +33,17 @@ int main() {
           for (int i = 0; i < n; ++i)
             if (std::llabs(v[i]) > ((int64_t)1 << (22 + span / 2))) v.push_back(-v[i]);
         __int128 exact = 0;
-        cisor::Fp32Sum a;
+        cisor::Fp32Sum part[8], a;  // as the warps of a CTA sum: eight sums in turn, added in order
         double d = 0, big = 0;
+        int i = 0;
         for (int64_t x : v) {
           const float f = std::ldexp((float)x, -40);  // exact: 24 significant bits
           exact += x;
-          a.add(f);
+          part[i++ % 8].add(f);
           d += f;
           big = std::fmax(big, std::fabs(f));
         }
+        for (const auto& p : part) a.add(p);
         // errors in units of 2^-40, exactly: the sums are multiples of it below 2^80, a double's part of them exact
         const auto err = [&](double s) {
           const double hi = std::ldexp(s, 40);
